@@ -1,0 +1,349 @@
+// mw_convolve_batched for series whose digits fit in shared memory: products of
+// truncated power series, c_i = sum_{k<=i} a_k b_{i-k} (Section 2's diagonal
+// sums s_i are these convolutions), the same words as one inner product per
+// coefficient (mw_dot.cu) gives.
+//
+// Coefficient i is cut on the grids of its own vectors: E_a(i), the largest
+// exponent of a_0..a_i, and E_b(i) likewise.  Both only grow with i, so the
+// coefficients fall into segments of equal (E_a, E_b), a few for ordinary series
+// (as many as there are new largest entries), and one cut of a_0..a_i1 and
+// b_0..b_i1 serves a segment's coefficients i0..i1.  A CTA works on one series:
+//   1. exponents of all entries (every word), prefix maxima, segment starts;
+//   2. per segment, the 24-bit balanced digits of the entries into shared memory
+//      (only those not cut yet on the same grid);
+//   3. a warp takes 32 consecutive coefficients (a row), one a lane: for every k
+//      the digits of a_k are read as a broadcast, those of b_{i-k} at consecutive
+//      addresses, and S^2/2 products go into int64 diagonal sums in registers
+//      (|d d| <= 2^46 and S n < 2^17 terms at most: far below 2^63);
+//   4. each lane fuses and rounds its own coefficient.
+// Row r has 32 (r + 1) steps, so a warp takes rows r and R - 1 - r; with few
+// series `ks` warps share a row's k and add their sums in shared memory.
+//
+// Bound by the 32 x 32 -> 64 bit multiply-adds.  One CTA per coefficient (which
+// cuts i + 1 entries of both series again for each) took 17.25 ms for 2,000
+// octo-double pairs of degree 127.
+#include <cuda.h>
+
+#include <algorithm>
+
+#include "mw_column.cuh"
+#include "mw_dot.cuh"
+
+namespace mw {
+namespace {
+
+constexpr int kSeriesWarps = 8;                    // most warps of a CTA
+constexpr size_t kSeriesSmem = 232448;             // shared memory a CTA can have
+
+template <int MW, int S> struct SeriesShape {
+  static constexpr int DC = S + kDotExtraD;
+  static constexpr int SP = (S + 3) / 4 * 4;       // a's digits of one entry, in int4
+  static constexpr int NL = 2 * ((kDotW * S + 3 + 127) / 128);
+  static constexpr int NL32 = (kDotW * (DC - 1) + 65 + 31) / 32;   // |X| < 2^(64 + w (D-1))
+  // column of a thread: the slots of cut_column (m >= 8), then the rounding's limbs
+  static constexpr int COL = (MW >= 8 && S + 3 > NL32) ? S + 3 : NL32;
+};
+
+__host__ __device__ inline int64_t series_round32(int64_t n) { return (n + 31) & ~(int64_t)31; }
+
+template <int MW, int S>
+size_t series_smem(int64_t n, int warps, int ks) {
+  using SH = SeriesShape<MW, S>;
+  const size_t nr = (size_t)series_round32(n);
+  return 4 * (nr * SH::SP + S * (nr + 32) + 2 * nr + nr + 32 + (size_t)SH::COL * 32 * warps) + 64 +
+         (size_t)(warps / ks) * (ks - 1) * SH::DC * 32 * 8;
+}
+
+template <int MW, int S>
+__global__ void __launch_bounds__(32 * kSeriesWarps, MW == 16 ? 1 : 2)
+    series_kernel(const DotArgs a, int ks, int pairs, int parts) {
+  using SH = SeriesShape<MW, S>;
+  constexpr int DC = SH::DC, SP = SH::SP, NL = SH::NL, NL32 = SH::NL32;
+  const int n = (int)a.K, nr = (int)series_round32(n), rows = nr / 32;
+  const int row_pairs = (rows + 1) / 2, nthr = blockDim.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  extern __shared__ int4 smem4[];
+  int64_t *red = reinterpret_cast<int64_t *>(smem4);           // [pairs][ks - 1][DC][32]
+  int32_t *da = reinterpret_cast<int32_t *>(red + (size_t)pairs * (ks - 1) * DC * 32);  // [nr][SP]
+  int32_t *db = da + (size_t)nr * SP;                          // [S][32 zeros, nr]
+  int32_t *pe = db + (size_t)S * (nr + 32);                    // prefix exponents [2][nr]
+  int32_t *segs = pe + 2 * nr;                                 // first coefficient of a segment
+  int32_t *flags = segs + nr + 32;         // [0] segments, [1..2] smallest exponents, [3] bits
+  uint32_t *col = reinterpret_cast<uint32_t *>(flags + 16) + tid;
+  const int ldb_ = nr + 32;
+  for (int t = tid; t < S * 32; t += nthr) db[(t >> 5) * ldb_ + (t & 31)] = 0;
+
+  for (int64_t task = blockIdx.x; task < a.count * parts; task += gridDim.x) {
+    const int64_t s_idx = task / parts;
+    const int part = (int)(task - s_idx * parts);
+    const double *px[2] = {a.A + s_idx * a.lda, a.B + s_idx * a.ldb};
+    const int64_t ps[2] = {a.psa, a.psb};
+    // 1. exponents
+    __syncthreads();                               // the previous task's flags were read
+    if (tid < 4) flags[tid] = tid == 3 ? 0 : -kExpZero;
+    __syncthreads();
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      int emin = -kExpZero;
+      for (int k = tid; k < nr; k += nthr) {
+        int e = kExpZero;
+        if (k < n) {
+          uint64_t mx = 0;                         // the entry's largest word
+#pragma unroll
+          for (int j = 0; j < MW; ++j) {
+            const uint64_t u = (uint64_t)__double_as_longlong(px[o][j * ps[o] + k]) & 0x7FFFFFFFFFFFFFFFull;
+            mx = u > mx ? u : mx;
+          }
+          e = exp_plus1(__longlong_as_double((long long)mx));
+          if (e == kExpNonFinite) {
+            atomicOr(&flags[3], MW_ENONFINITE);
+            e = kExpZero;
+          }
+          if (e != kExpZero) emin = min(emin, e);
+        }
+        pe[o * nr + k] = e;
+      }
+      if (emin != -kExpZero) atomicMin(&flags[1 + o], emin);
+    }
+    __syncthreads();
+    if (warp == 0) {                               // prefix maxima and segment starts
+      int carry[2] = {kExpZero, kExpZero}, nseg = 0;
+      for (int k0 = 0; k0 < nr; k0 += 32) {
+        bool first = k0 + lane == 0;
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+          int e = max(pe[o * nr + k0 + lane], carry[o]);
+          for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, e, d);
+            if (lane >= d) e = max(e, y);
+          }
+          pe[o * nr + k0 + lane] = e;
+          int before = __shfl_up_sync(0xffffffffu, e, 1);
+          if (lane == 0) before = carry[o];
+          first |= before != e;
+          carry[o] = __shfl_sync(0xffffffffu, e, 31);
+        }
+        first &= k0 + lane < n;
+        const unsigned m = __ballot_sync(0xffffffffu, first);
+        if (first) segs[nseg + __popc(m & ((1u << lane) - 1u))] = k0 + lane;
+        nseg += __popc(m);
+      }
+      if (lane == 0) {
+        segs[nseg] = n;
+        flags[0] = nseg;
+        const int ma = carry[0], mb = carry[1];
+        const int sa = ma == kExpZero ? 0 : ma - flags[1], sb = mb == kExpZero ? 0 : mb - flags[2];
+        if ((a.range_A >= 0 && sa > a.range_A) || (a.range_B >= 0 && sb > a.range_B))
+          raise_status(a.status, MW_WRANGE);
+        if (flags[3]) raise_status(a.status, (unsigned)flags[3]);
+      }
+    }
+    __syncthreads();
+    const int nseg = flags[0];
+    const int rp = part * pairs + warp / ks, kw = warp - (warp / ks) * ks;
+    // entries 0 .. done[o] - 1 hold digits on the grid of exponent cutE[o]
+    int done[2] = {0, 0}, cutE[2] = {0, 0};
+    for (int g = 0; g < nseg; ++g) {
+      const int i0 = segs[g], i1 = segs[g + 1] - 1;
+      // the rows of this CTA's pairs that the segment touches
+      const int r0 = i0 >> 5, r1 = i1 >> 5;
+      const int plo = part * pairs, phi = min(plo + pairs, row_pairs) - 1;
+      const int lo_max = min(phi, r1), hi_max = min(rows - 1 - plo, r1);   // largest row touched
+      const bool lo_in = lo_max >= plo && lo_max >= r0;
+      const bool hi_in = hi_max >= rows - 1 - phi && hi_max >= r0;
+      if (!lo_in && !hi_in) continue;
+      const int kmax = min(i1, 32 * (hi_in ? hi_max : lo_max) + 31);
+      const int E[2] = {pe[i0] == kExpZero ? 0 : pe[i0], pe[nr + i0] == kExpZero ? 0 : pe[nr + i0]};
+      __syncthreads();                             // the previous segment's digits were read
+      // 2. digits
+      if constexpr (MW >= 8)
+        for (int c = 0; c < S + 3; ++c) col[c * nthr] = 0u;    // cut_column leaves it zero
+      const int base[2] = {cutE[0] == E[0] ? done[0] : 0, cutE[1] == E[1] ? done[1] : 0};
+      const int na = max(kmax + 1 - base[0], 0), nb = max(kmax + 1 - base[1], 0);
+      bool ok = true;
+      for (int u = tid; u < na + nb; u += nthr) {
+        const int o = u >= na, k = o ? base[1] + u - na : base[0] + u;
+        const double *p = (o ? px[1] : px[0]) + k;
+        const int64_t pst = o ? ps[1] : ps[0];
+        const int F = kDotW * S - 2 - (o ? E[1] : E[0]);
+        double x[MW];
+#pragma unroll
+        for (int j = 0; j < MW; ++j) x[j] = p[j * pst];
+        // digit p of entry k: a's at da[k SP + p], b's at db[p (nr + 32) + 32 + k]
+        int32_t *dst = o ? db + 32 + k : da + k * SP;
+        const int step = o ? ldb_ : 1;
+        if constexpr (MW >= 8) {
+          ok &= cut_column<MW, kDotW>(x, F, S, col, nthr,
+                                      [&](int q, int32_t d) { dst[(S - 1 - q) * step] = d; });
+        } else {
+          uint64_t T[NL];
+          int32_t d[S];
+          fixed_point<MW, NL>(x, F, T);
+          ok &= dot_digits<S, NL>(T, d);
+#pragma unroll
+          for (int q = 0; q < S; ++q) dst[q * step] = d[q];
+        }
+      }
+      if (!ok) raise_status(a.status, MW_ERANGE);
+      done[0] = max(kmax + 1, base[0]);
+      done[1] = max(kmax + 1, base[1]);
+      cutE[0] = E[0];
+      cutE[1] = E[1];
+      __syncthreads();
+      // 3. diagonal sums of rows rp and rows - 1 - rp
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        const int r = half ? rows - 1 - rp : rp;
+        const bool mine = rp < row_pairs && !(half && r == rp) && r >= r0 && r <= r1;
+        const int i = 32 * r + lane;
+        int64_t s[DC];
+#pragma unroll
+        for (int t = 0; t < DC; ++t) s[t] = 0;
+        if (mine) {
+          const int kend = min(i1, 32 * r + 31);
+#pragma unroll 1
+          for (int k = kw; k <= kend; k += ks) {
+            int32_t x[SP], y[S];
+            const int4 *xa = reinterpret_cast<const int4 *>(da + k * SP);
+#pragma unroll
+            for (int q = 0; q < SP / 4; ++q) {
+              const int4 v = xa[q];
+              x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
+            }
+            const int32_t *yb = db + 32 + i - k;   // zero for i < k
+#pragma unroll
+            for (int q = 0; q < S; ++q) y[q] = yb[q * ldb_];
+#pragma unroll
+            for (int p = 0; p < S; ++p)
+#pragma unroll
+              for (int q = 0; q < S - p; ++q) s[p + q] += (int64_t)x[p] * (int64_t)y[q];
+#pragma unroll
+            for (int t = S; t < DC; ++t)
+              if (t < a.D) {
+#pragma unroll
+                for (int p = t - S + 1; p < S; ++p) s[t] += (int64_t)x[p] * (int64_t)y[t - p];
+              }
+          }
+        }
+        if (ks > 1) {
+          int64_t *rd = red + (size_t)(warp / ks) * (ks - 1) * DC * 32 + lane;
+          if (kw > 0 && mine)
+#pragma unroll
+            for (int t = 0; t < DC; ++t) rd[((kw - 1) * DC + t) * 32] = s[t];
+          __syncthreads();
+          if (kw == 0 && mine)
+            for (int w = 1; w < ks; ++w)
+#pragma unroll
+              for (int t = 0; t < DC; ++t) s[t] += rd[((w - 1) * DC + t) * 32];
+        }
+        // 4. fusion and rounding: X = sum_t s_t 2^(w (DC-1-t)) in 24-bit fields from
+        // the least significant end, joined into 32-bit limbs (diagonals D.. are zero)
+        if (mine && kw == 0) {
+          uint32_t f[DC + 4];
+          int64_t carry = 0;
+#pragma unroll
+          for (int j = 0; j < DC; ++j) {
+            if (DC - 1 - j < a.D) carry += s[DC - 1 - j];
+            f[j] = (uint32_t)carry & 0xFFFFFFu;
+            carry >>= 24;
+          }
+#pragma unroll
+          for (int j = DC; j < DC + 4; ++j) {
+            f[j] = (uint32_t)carry & 0xFFFFFFu;
+            carry >>= 24;
+          }
+          uint32_t U[NL32];
+#pragma unroll
+          for (int l = 0; l < NL32; ++l) {
+            const int j = 32 * l / 24, o = 32 * l % 24;
+            static_assert((32 * (NL32 - 1)) / 24 + 2 < DC + 4, "fields cover the limbs");
+            uint32_t v = (f[j] >> o) | (f[j + 1] << (24 - o));
+            if (48 - o < 32) v |= f[j + 2] << (48 - o);
+            U[l] = v;
+          }
+          if (i >= i0 && i <= i1) {
+            double *c = a.C + s_idx * a.ldc + i;
+            const int64_t psc = a.psc;
+            round_column<MW, NL32>(U, col, nthr, E[0] + E[1] + 4 - kDotW * (DC + 1),
+                                   [&](int w, double v) { c[w * psc] = v; });
+          }
+        }
+        if (ks > 1) __syncthreads();               // red and the columns are reused
+      }
+    }
+  }
+}
+
+template <int MW, int S>
+int launch_series_s(const DotArgs &a, cudaStream_t st) {
+  static bool attr_set = false;   // once per instance
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(series_kernel<MW, S>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSeriesSmem);
+    if (e != cudaSuccess) return cuda_fail(e, "series kernel smem attribute");
+    attr_set = true;
+  }
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int row_pairs = (int)((a.K + 63) / 64);
+  // warps sharing a row's k: more while the rows of all series leave SMs with
+  // fewer than eight warps
+  int ks = 1;
+  while (ks < kSeriesWarps && a.count * row_pairs * ks < (int64_t)8 * nsm) ks *= 2;
+  int pairs = std::min(row_pairs, kSeriesWarps / ks);
+  while (pairs > 1 && series_smem<MW, S>(a.K, pairs * ks, ks) > kSeriesSmem) --pairs;
+  while (ks > 1 && series_smem<MW, S>(a.K, pairs * ks, ks) > kSeriesSmem) ks /= 2;
+  const size_t smem = series_smem<MW, S>(a.K, pairs * ks, ks);
+  if (smem > kSeriesSmem) return fail(MW_EUNSUPPORTED, "series of %lld coefficients", (long long)a.K);
+  const int parts = (row_pairs + pairs - 1) / pairs;
+  const unsigned grid = (unsigned)std::min<int64_t>(a.count * parts, 1 << 30);
+  series_kernel<MW, S><<<grid, 32 * pairs * ks, smem, st>>>(a, ks, pairs, parts);
+  return cuda_fail(cudaGetLastError(), "series kernel launch");
+}
+
+template <int MW, int S>
+int launch_series_m(int s_req, const DotArgs &a, cudaStream_t st) {
+  if constexpr (S > DotS<MW>::hi) {
+    return fail(MW_EUNSUPPORTED, "series need %d pieces, at most %d supported", s_req,
+                DotS<MW>::hi);
+  } else {
+    if (s_req == S) return launch_series_s<MW, S>(a, st);
+    return launch_series_m<MW, S + 1>(s_req, a, st);
+  }
+}
+
+template <int MW, int S>
+bool series_fits_m(int s_req, int64_t n) {
+  if constexpr (S > DotS<MW>::hi) {
+    return false;
+  } else {
+    if (s_req == S) return n <= 4096 && series_smem<MW, S>(n, 1, 1) <= kSeriesSmem;
+    return series_fits_m<MW, S + 1>(s_req, n);
+  }
+}
+
+}  // namespace
+
+bool series_fits(int m, int S, int64_t n) {
+  switch (m) {
+    case 2: return series_fits_m<2, DotS<2>::lo>(S, n);
+    case 4: return series_fits_m<4, DotS<4>::lo>(S, n);
+    case 8: return series_fits_m<8, DotS<8>::lo>(S, n);
+    case 16: return series_fits_m<16, DotS<16>::lo>(S, n);
+  }
+  return false;
+}
+
+int launch_series(int m, int S, const DotArgs &a, cudaStream_t st) {
+  switch (m) {
+    case 2: return launch_series_m<2, DotS<2>::lo>(S, a, st);
+    case 4: return launch_series_m<4, DotS<4>::lo>(S, a, st);
+    case 8: return launch_series_m<8, DotS<8>::lo>(S, a, st);
+    case 16: return launch_series_m<16, DotS<16>::lo>(S, a, st);
+  }
+  return fail(MW_EINVAL, "m must be 2, 4, 8 or 16");
+}
+
+}  // namespace mw
