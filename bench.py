@@ -990,13 +990,19 @@ def run_series(args, mw, torch, dist, rank, world, dev):
     return line
 
 
-# FP64 instructions of one m-double operation on the GPU path (two_sum 6,
-# fast_two_sum 3, two_prod 2 = a multiply and a fused multiply-add, a plain add or
-# multiply 1, a division counted as 1), generic operands (every term nonzero), by
-# stepping through the algorithms of mw_elementwise
+# FP64 instructions of one m-double operation of the textbook algorithms (Knuth's
+# two_sum 6, fast_two_sum 3, two_prod 2 = a multiply and a fused multiply-add, a
+# plain add or multiply 1, a division counted as 1), generic operands (every term
+# nonzero), by stepping through the oracle's algorithms
 ELEMENTWISE_FP64_OPS = {2: {"add": 20, "mul": 9, "div": 79},
                         4: {"add": 132, "mul": 515, "div": 2797},
                         8: {"add": 552, "mul": 3655, "div": 35225}}
+# The FP64 instructions mw_elementwise issues for them: two_sum 3 (operands ordered
+# on the integer units), sums only in the last sweep of a renormalisation, no
+# products with the zero words of a quotient word.  What its roofline counts.
+ELEMENTWISE_GPU_FP64 = {2: {"add": 14, "mul": 9, "div": 52},
+                        4: {"add": 58, "mul": 231, "div": 601},
+                        8: {"add": 260, "mul": 1725, "div": 5075}}
 
 
 def run_elementwise(args, mw, torch, dist, rank, world, dev):
@@ -1030,7 +1036,7 @@ def run_elementwise(args, mw, torch, dist, rank, world, dev):
     step_ms, _, clk = timed(step, args.steps, flush, mw, dist, dev, phase=False)
     value, t_step = aggregate(sum(step_ms) / 1e3, n, args.steps, dist, dev)   # G entries/s
     kern_s = statistics.mean(step_ms) / 1e3
-    ops = ELEMENTWISE_FP64_OPS[m][op]
+    ops = ELEMENTWISE_GPU_FP64[m][op]
     achieved = ops * n / kern_s / 1e12
     peak = fp64_peak / 2
     _, _, hbm_gbs, hbm_src = load_peaks()

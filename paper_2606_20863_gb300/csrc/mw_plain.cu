@@ -16,19 +16,12 @@
 // thread (ty, tx) the outputs (ty + 16 a, tx + 16 b); pieces are staged in
 // shared memory 16 columns of the reduction at a time.
 #include "mw_device.cuh"
+#include "mw_eft.cuh"
 
 namespace mw {
 namespace {
 
 constexpr int BKP = 16;
-
-__device__ __forceinline__ double two_sum(double a, double b, double &e) {
-  const double s = __dadd_rn(a, b);
-  const double bv = __dsub_rn(s, a);
-  const double av = __dsub_rn(s, bv);
-  e = __dadd_rn(__dsub_rn(a, av), __dsub_rn(b, bv));
-  return s;
-}
 
 // Add x into the (W)-word accumulator s: top-down two-sum cascade (the error of
 // each word moves to the next, the last rounding error is dropped), then a

@@ -2,8 +2,8 @@
 // vectorized (error-free summation) one against: every term a_ik b_kj is an
 // m-double multiplication followed by an m-double addition into the running sum,
 // k in order, built from the error-free transformations of floating-point
-// arithmetic (Section 1's multiword arithmetic):
-//   two_sum (Knuth): s = fl(a + b), e = a + b - s exactly;
+// arithmetic (Section 1's multiword arithmetic; mw_eft.cuh):
+//   two_sum: s = fl(a + b), e = a + b - s exactly;
 //   fast_two_sum (Dekker): the same for |a| >= |b|;
 //   two_prod: p = fl(a b), e = a b - p exactly (one fused multiply-add; the
 //     same p and e as Dekker's splitting, which needs no fma).
@@ -18,7 +18,8 @@
 // contracted into a multiply-add.
 //
 // One thread per output, 16 x 16 outputs a CTA, 16-wide k panels of A and B
-// staged in shared memory (m planes each).  The FP64 pipe bounds it.
+// staged in shared memory (m planes each).  The FP64 pipe bounds it (2 lanes a
+// clock and SM): what a kernel here costs is its FP64 instructions.
 //
 // The same operations serve mw_elementwise (Table 1's add, mul and div entry by
 // entry).  Division is long division, the paper giving only its operation count:
@@ -33,30 +34,13 @@
 #include <algorithm>
 
 #include "mw_device.cuh"
+#include "mw_eft.cuh"
 #include "mw_internal.h"
 
 namespace mw {
 namespace {
 
 constexpr int kTT = 16;   // outputs per CTA side, k per panel
-
-__device__ __forceinline__ double tb_two_sum(double a, double b, double &e) {
-  const double s = __dadd_rn(a, b);
-  const double bv = __dsub_rn(s, a);
-  const double av = __dsub_rn(s, bv);
-  e = __dadd_rn(__dsub_rn(a, av), __dsub_rn(b, bv));
-  return s;
-}
-__device__ __forceinline__ double tb_fast_two_sum(double a, double b, double &e) {
-  const double s = __dadd_rn(a, b);
-  e = __dsub_rn(b, __dsub_rn(s, a));
-  return s;
-}
-__device__ __forceinline__ double tb_two_prod(double a, double b, double &e) {
-  const double p = __dmul_rn(a, b);
-  e = __fma_rn(a, b, -p);
-  return p;
-}
 
 // n terms in level order -> m words: sweep j sums x[0..n-1-j] bottom-up; its top
 // sum is word j, its rounding errors the terms of sweep j + 1.
@@ -73,7 +57,7 @@ __device__ __forceinline__ void tb_renorm(double (&x)[N], double (&r)[M]) {
 #pragma unroll
     for (int i = n - 2; i >= 0; --i) {
       double e;
-      s = tb_two_sum(x[i], s, e);
+      s = two_sum(x[i], s, e);
       x[i + 1] = e;
     }
     r[j] = s;
@@ -86,12 +70,12 @@ template <int M>
 __device__ __forceinline__ void tb_add(const double (&a)[M], const double (&b)[M], double (&r)[M]) {
   if constexpr (M == 2) {
     double e, f;
-    double s = tb_two_sum(a[0], b[0], e);
-    const double t = tb_two_sum(a[1], b[1], f);
+    double s = two_sum(a[0], b[0], e);
+    const double t = two_sum(a[1], b[1], f);
     e = __dadd_rn(e, t);
-    s = tb_fast_two_sum(s, e, e);
+    s = fast_two_sum(s, e, e);
     e = __dadd_rn(e, f);
-    s = tb_fast_two_sum(s, e, e);
+    s = fast_two_sum(s, e, e);
     r[0] = s;
     r[1] = e;
   } else {
@@ -109,9 +93,9 @@ template <int M>
 __device__ __forceinline__ void tb_mul(const double (&a)[M], const double (&b)[M], double (&r)[M]) {
   if constexpr (M == 2) {
     double e;
-    double p = tb_two_prod(a[0], b[0], e);
+    double p = two_prod(a[0], b[0], e);
     e = __dadd_rn(e, __dadd_rn(__dmul_rn(a[0], b[1]), __dmul_rn(a[1], b[0])));
-    p = tb_fast_two_sum(p, e, e);
+    p = fast_two_sum(p, e, e);
     r[0] = p;
     r[1] = e;
   } else {
@@ -125,7 +109,7 @@ __device__ __forceinline__ void tb_mul(const double (&a)[M], const double (&b)[M
 #pragma unroll
     for (int l = 0; l < M; ++l) {
 #pragma unroll
-      for (int i = 0; i <= l; ++i) t[n++] = tb_two_prod(a[i], b[l - i], lo_cur[i]);
+      for (int i = 0; i <= l; ++i) t[n++] = two_prod(a[i], b[l - i], lo_cur[i]);
 #pragma unroll
       for (int i = 0; i < l; ++i) t[n++] = lo_prev[i];
 #pragma unroll
@@ -139,6 +123,33 @@ __device__ __forceinline__ void tb_mul(const double (&a)[M], const double (&b)[M
   }
 }
 
+// The product of (q, 0, ..., 0) and b: tb_mul without the terms that are exact
+// zeros.  A zero term leaves every sum of a sweep as it is and its own error is
+// zero, so the words are the same.
+template <int M>
+__device__ __forceinline__ void tb_mul_word(double q, const double (&b)[M], double (&r)[M]) {
+  if constexpr (M == 2) {
+    double e;
+    double p = two_prod(q, b[0], e);
+    e = __dadd_rn(e, __dmul_rn(q, b[1]));
+    p = fast_two_sum(p, e, e);
+    r[0] = p;
+    r[1] = e;
+  } else {
+    double t[2 * M], lo = 0.0;
+#pragma unroll
+    for (int l = 0; l < M; ++l) {
+      double e;
+      const double p = two_prod(q, b[l], e);
+      t[l ? 2 * l - 1 : 0] = p;
+      if (l) t[2 * l] = lo;
+      lo = e;
+    }
+    t[2 * M - 1] = lo;
+    tb_renorm<M, 2 * M>(t, r);
+  }
+}
+
 template <int M>
 __device__ __forceinline__ void tb_div(const double (&a)[M], const double (&b)[M], double (&r)[M]) {
   double rem[M], q[M + 1];
@@ -148,11 +159,8 @@ __device__ __forceinline__ void tb_div(const double (&a)[M], const double (&b)[M
   for (int i = 0; i <= M; ++i) {
     q[i] = __ddiv_rn(rem[0], b[0]);
     if (i == M) break;
-    double qv[M], t[M], s[M];
-    qv[0] = q[i];
-#pragma unroll
-    for (int w = 1; w < M; ++w) qv[w] = 0.0;
-    tb_mul<M>(qv, b, t);
+    double t[M], s[M];
+    tb_mul_word<M>(q[i], b, t);
 #pragma unroll
     for (int w = 0; w < M; ++w) t[w] = -t[w];
     tb_add<M>(rem, t, s);
@@ -167,7 +175,9 @@ __device__ __forceinline__ void tb_div(const double (&a)[M], const double (&b)[M
 }
 
 // C = A op B entry by entry (OP 0 add, 1 mul, 2 div), n entries, m planes each;
-// one thread per entry, the loads of a plane coalesced.
+// one thread per entry, the loads of a plane coalesced.  Quad-double mul of 2^22
+// entries: 3,330 us with Knuth's two_sum (six FP64 additions), 1,830 us with
+// operands ordered on the integer units (three).
 template <int MW, int OP>
 __global__ void __launch_bounds__(256) elementwise_kernel(const double *__restrict__ A,
                                                           int64_t psa,
