@@ -488,7 +488,7 @@ int mw_gemm(const mw_plan *plan, int transA, int transB, int64_t M, int64_t N, i
   if (p.mode == MW_PLAIN) {
     PlainArgs a{};
     a.m = p.m; a.w = p.w; a.S_A = p.S_A; a.S_B = p.S_B; a.D = p.D;
-    a.M = M; a.N = N; a.Kp = L.Kp;
+    a.M = M; a.N = N; a.K = K; a.Kp = L.Kp;
     a.dA = reinterpret_cast<const double *>(w8 + L.digA);
     a.dB = reinterpret_cast<const double *>(w8 + L.digB);
     a.eA = o.eA; a.eB = o.eB; a.C = C; a.ldc = ldc; a.psc = psc;

@@ -39,7 +39,7 @@ int launch_split(const SplitArgs &a, bool exponents_only, cudaStream_t s);
 // ---- plain FP64 form (mw_plain.cu) -------------------------------------------
 struct PlainArgs {
   int m, w, S_A, S_B, D;
-  int64_t M, N, Kp;            // Kp: padded reduction length (digit row stride)
+  int64_t M, N, K, Kp;         // Kp: padded reduction length (digit row stride)
   const double *dA, *dB;        // S_A x M x Kp, S_B x N x Kp pieces
   const int32_t *eA, *eB;       // row / column exponents
   double *C;

@@ -14,7 +14,9 @@
 //
 // Tiling: a block of 16 x 16 threads computes a (16 TH) x (16 TH) tile of C,
 // thread (ty, tx) the outputs (ty + 16 a, tx + 16 b); pieces are staged in
-// shared memory 16 columns of the reduction at a time.
+// shared memory 16 columns of the reduction at a time.  This kernel takes any
+// plan; plain_split_kernel below (4 x 8 outputs a CTA) is faster at every size and
+// takes the plans whose pieces fit in its shared memory.
 #include "mw_device.cuh"
 #include "mw_eft.cuh"
 
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(256, 1) plain_kernel(PlainArgs a) {
       const int q = t - p;
       const double *pa = a.dA + (int64_t)p * a.M * a.Kp;
       const double *pb = a.dB + (int64_t)q * a.N * a.Kp;
-      for (int64_t k0 = 0; k0 < a.Kp; k0 += BKP) {
+      for (int64_t k0 = 0; k0 < a.K; k0 += BKP) {       // zeros from K up
 #pragma unroll
         for (int r = 0; r < TH; ++r) {
           const int row = lr + 16 * r;
@@ -138,8 +140,96 @@ __global__ void __launch_bounds__(256, 1) plain_kernel(PlainArgs a) {
     }
 }
 
+// 4 x 8 outputs a CTA.  The FP64 pipe takes 2 multiply-adds a clock and SM, so
+// loads need no reuse in registers; what counts is that every SM has its share of
+// the work.  A lane holds one output and the CTA's 8 warps take every eighth k of a
+// chunk of KC (all pieces of the chunk's 4 rows and 8 columns in shared memory,
+// rows KC + 2 apart: lanes read distinct banks or the same word).  Every partial
+// diagonal sum is exact, so the warps' sums add up to the same s_t in any order;
+// warp 0 then adds the s_t into the m-double accumulator, t in order, as
+// plain_kernel does.  plain_kernel against this one, us (FP64 floor): dd 64^3
+// 1,520 / 47 (9), dd 384^3 10,290 / 2,530 (2,420), qd 640^3 37,390 / 33,080
+// (32,770), od 256^3 17,380 / 8,010 (6,930).
+constexpr int SR = 4, SC = 8, SWARPS = 8;
+
+inline size_t plain_split_smem(int S_A, int S_B, int D, int KC) {
+  return 8 * ((size_t)(SR * S_A + SC * S_B) * (KC + 2) + (size_t)SWARPS * D * 32);
+}
+
+template <int MW>
+__global__ void __launch_bounds__(32 * SWARPS) plain_split_kernel(PlainArgs a, int KC) {
+  extern __shared__ double sm[];
+  const int LD = KC + 2;
+  double *As = sm, *Bs = As + SR * a.S_A * LD, *st = Bs + SC * a.S_B * LD;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r = lane >> 3, c = lane & 7;
+  const int64_t tiles_n = (a.N + SC - 1) / SC, ti = blockIdx.x / tiles_n;
+  const int64_t i0 = ti * SR, j0 = (blockIdx.x - ti * tiles_n) * SC;
+  for (int64_t k0 = 0; k0 < a.K; k0 += KC) {
+    const int kc = (int)(a.K - k0 < KC ? (a.K - k0 + 7) & ~(int64_t)7 : KC);   // zeros from K up
+    if (k0) __syncthreads();                       // the previous chunk was read
+    for (int u = warp; u < SR * a.S_A; u += SWARPS) {
+      const int64_t i = i0 + (u & (SR - 1));
+      const double *src = a.dA + ((int64_t)(u / SR) * a.M + i) * a.Kp + k0;
+      for (int k = lane; k < kc; k += 32) As[u * LD + k] = i < a.M ? src[k] : 0.0;
+    }
+    for (int u = warp; u < SC * a.S_B; u += SWARPS) {
+      const int64_t j = j0 + (u & (SC - 1));
+      const double *src = a.dB + ((int64_t)(u / SC) * a.N + j) * a.Kp + k0;
+      for (int k = lane; k < kc; k += 32) Bs[u * LD + k] = j < a.N ? src[k] : 0.0;
+    }
+    __syncthreads();
+    for (int t = 0; t < a.D; ++t) {
+      const int plo = max(0, t - a.S_B + 1), phi = min(t, a.S_A - 1);
+      double acc = k0 ? st[(warp * a.D + t) * 32 + lane] : 0.0;
+      for (int p = plo; p <= phi; ++p) {
+        const double *x = As + (p * SR + r) * LD, *y = Bs + ((t - p) * SC + c) * LD;
+#pragma unroll 4
+        for (int k = warp; k < kc; k += SWARPS) acc = __fma_rn(x[k], y[k], acc);
+      }
+      st[(warp * a.D + t) * 32 + lane] = acc;
+    }
+  }
+  __syncthreads();
+  for (int t = warp; t < a.D; t += SWARPS) {       // the warps' sums of s_t into warp 0's
+    double v = st[t * 32 + lane];
+#pragma unroll
+    for (int w = 1; w < SWARPS; ++w) v = __dadd_rn(v, st[(w * a.D + t) * 32 + lane]);
+    st[t * 32 + lane] = v;
+  }
+  __syncthreads();
+  const int64_t i = i0 + r, j = j0 + c;
+  if (warp || i >= a.M || j >= a.N) return;
+  double acc[MW + 1], out[MW];
+#pragma unroll
+  for (int w = 0; w <= MW; ++w) acc[w] = 0.0;
+  const int e = a.eA[i] + a.eB[j] + 4;
+  for (int t = 0; t < a.D; ++t) accumulate<MW + 1>(acc, scalbn(st[t * 32 + lane], e - a.w * (t + 2)));
+  renormalize<MW + 1, MW>(acc, out);
+#pragma unroll
+  for (int w = 0; w < MW; ++w) a.C[w * a.psc + i * a.ldc + j] = out[w];
+}
+
 template <int MW, int TH>
 int launch(const PlainArgs &a, cudaStream_t s) {
+  // the longest chunk that leaves room for 3 CTAs an SM, from 32 on for 2 (many
+  // pieces: short chunks cost more than the third CTA gives)
+  int KC = 64;
+  while (KC > 32 && plain_split_smem(a.S_A, a.S_B, a.D, KC) > 75776) KC -= 16;
+  while (KC > 8 && plain_split_smem(a.S_A, a.S_B, a.D, KC) > 115712) KC -= 8;
+  const size_t smem = plain_split_smem(a.S_A, a.S_B, a.D, KC);
+  const int64_t tiles = (a.N + SC - 1) / SC * ((a.M + SR - 1) / SR);
+  if (smem <= 232448 && tiles <= 0x7fffffff) {
+    static bool attr_set = false;   // once per instance
+    if (!attr_set) {
+      cudaError_t e = cudaFuncSetAttribute(plain_split_kernel<MW>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+      if (e != cudaSuccess) return cuda_fail(e, "plain kernel smem attribute");
+      attr_set = true;
+    }
+    plain_split_kernel<MW><<<(unsigned)tiles, 32 * SWARPS, smem, s>>>(a, KC);
+    return cuda_fail(cudaGetLastError(), "plain kernel launch");
+  }
   constexpr int BT = 16 * TH;
   dim3 grid((unsigned)((a.N + BT - 1) / BT), (unsigned)((a.M + BT - 1) / BT));
   plain_kernel<MW, TH><<<grid, 256, 0, s>>>(a);
