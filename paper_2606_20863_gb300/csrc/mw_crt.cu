@@ -66,13 +66,14 @@ constexpr bool all_odd() {
 static_assert(all_odd(), "the moduli must be odd and at most 513");
 constexpr int kPow16 = 65;   // 2^(16 j) mod p for j = 0..64 (T of up to 16 64-bit limbs)
 
-// Per modulus: p, floor(2^32 / p) for reducing 32-bit values, p and 1/p in
-// float (table entries, so that no conversion instruction runs per residue),
-// and 2^(16 j) mod p.
+// Per modulus: p, floor(2^32 / p) for reducing 32-bit values, 1/p and -p of two
+// neighbouring moduli as packed floats (table entries, so that no conversion
+// instruction runs per residue), and 2^(16 j) mod p.
 struct CrtTab {
   uint32_t p[kCrtMaxModuli];
   uint32_t m32[kCrtMaxModuli];
-  float pf[kCrtMaxModuli], rcp[kCrtMaxModuli];
+  alignas(8) float rcp[kCrtMaxModuli];
+  alignas(8) float npf[kCrtMaxModuli];
   uint32_t pow16[kCrtMaxModuli][kPow16];
 };
 constexpr CrtTab make_crt_tab() {
@@ -81,7 +82,7 @@ constexpr CrtTab make_crt_tab() {
     const uint32_t p = kModuli[i];
     t.p[i] = p;
     t.m32[i] = (uint32_t)((1ull << 32) / p);
-    t.pf[i] = (float)p;
+    t.npf[i] = -(float)p;
     t.rcp[i] = 1.0f / (float)p;
     uint32_t x = 1u % p;
     for (int j = 0; j < kPow16; ++j) {
@@ -104,36 +105,172 @@ __device__ __forceinline__ int balanced(uint32_t r, uint32_t p) {
   return r >= p - (p >> 1) ? (int)r - (int)p : (int)r;
 }
 
-// The balanced residue of an exactly represented float integer z (|z| < 2^22)
-// modulo an odd p, in [-floor(p/2), floor(p/2)]: z - q p with q the nearest
-// integer to z / p.  fmaf(z, 1/p, 1.5 2^23) rounds the exact product z fl(1/p)
-// to an integer; that product differs from z / p by less than |z| 2^-24 / p <
-// 1 / (4p), while an integer z over an odd p lies at least 1 / (2p) from any
-// half integer, so q is the nearest integer to z / p itself.  Every step is
-// exact (|q p| < 2^23).
-__device__ __forceinline__ float balanced_f(float z, int t) {
-  const float q = fmaf(z, kCrt.rcp[t], 12582912.0f) - 12582912.0f;
-  return fmaf(-q, kCrt.pf[t], z);
-}
-
-// bfloat16 bits of an integer-valued float of magnitude at most 256 (at most 8
-// significant bits): its top 16 bits.
-__device__ __forceinline__ uint16_t bf16_bits_small(float r) {
-  return (uint16_t)(__float_as_uint(r) >> 16);
-}
-
-// T in [-2^(L-1), 2^(L-1)): every bit from L-1 up equals the sign.
+// T += y + (s & 1) on NL limbs, s zero or all ones: one carry chain.
 template <int NL>
-__device__ __forceinline__ bool in_range_bits(const uint64_t (&T)[NL], int L) {
-  const int b = L - 1, lb = b >> 6, ob = b & 63;
-  int64_t v = 0;
+__device__ __forceinline__ void add_limbs32(uint32_t (&T)[NL], const uint32_t (&y)[NL], uint32_t s);
+template <>
+__device__ __forceinline__ void add_limbs32<4>(uint32_t (&T)[4], const uint32_t (&y)[4], uint32_t s) {
+  asm("{\n" ".reg .u32 c;\n"
+      "add.cc.u32 c, %8, %8;\n"
+      "addc.cc.u32 %0, %0, %4;\n"
+      "addc.cc.u32 %1, %1, %5;\n"
+      "addc.cc.u32 %2, %2, %6;\n"
+      "addc.u32 %3, %3, %7;\n" "}"
+      : "+r"(T[0]), "+r"(T[1]), "+r"(T[2]), "+r"(T[3])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(s));
+}
+template <>
+__device__ __forceinline__ void add_limbs32<5>(uint32_t (&T)[5], const uint32_t (&y)[5], uint32_t s) {
+  asm("{\n" ".reg .u32 c;\n"
+      "add.cc.u32 c, %10, %10;\n"
+      "addc.cc.u32 %0, %0, %5;\n"
+      "addc.cc.u32 %1, %1, %6;\n"
+      "addc.cc.u32 %2, %2, %7;\n"
+      "addc.cc.u32 %3, %3, %8;\n"
+      "addc.u32 %4, %4, %9;\n" "}"
+      : "+r"(T[0]), "+r"(T[1]), "+r"(T[2]), "+r"(T[3]), "+r"(T[4])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(s));
+}
+template <>
+__device__ __forceinline__ void add_limbs32<6>(uint32_t (&T)[6], const uint32_t (&y)[6], uint32_t s) {
+  asm("{\n" ".reg .u32 c;\n"
+      "add.cc.u32 c, %12, %12;\n"
+      "addc.cc.u32 %0, %0, %6;\n"
+      "addc.cc.u32 %1, %1, %7;\n"
+      "addc.cc.u32 %2, %2, %8;\n"
+      "addc.cc.u32 %3, %3, %9;\n"
+      "addc.cc.u32 %4, %4, %10;\n"
+      "addc.u32 %5, %5, %11;\n" "}"
+      : "+r"(T[0]), "+r"(T[1]), "+r"(T[2]), "+r"(T[3]), "+r"(T[4]), "+r"(T[5])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(s));
+}
+template <>
+__device__ __forceinline__ void add_limbs32<7>(uint32_t (&T)[7], const uint32_t (&y)[7], uint32_t s) {
+  asm("{\n" ".reg .u32 c;\n"
+      "add.cc.u32 c, %14, %14;\n"
+      "addc.cc.u32 %0, %0, %7;\n"
+      "addc.cc.u32 %1, %1, %8;\n"
+      "addc.cc.u32 %2, %2, %9;\n"
+      "addc.cc.u32 %3, %3, %10;\n"
+      "addc.cc.u32 %4, %4, %11;\n"
+      "addc.cc.u32 %5, %5, %12;\n"
+      "addc.u32 %6, %6, %13;\n" "}"
+      : "+r"(T[0]), "+r"(T[1]), "+r"(T[2]), "+r"(T[3]), "+r"(T[4]), "+r"(T[5]), "+r"(T[6])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(s));
+}
+template <>
+__device__ __forceinline__ void add_limbs32<8>(uint32_t (&T)[8], const uint32_t (&y)[8], uint32_t s) {
+  asm("{\n" ".reg .u32 c;\n"
+      "add.cc.u32 c, %16, %16;\n"
+      "addc.cc.u32 %0, %0, %8;\n"
+      "addc.cc.u32 %1, %1, %9;\n"
+      "addc.cc.u32 %2, %2, %10;\n"
+      "addc.cc.u32 %3, %3, %11;\n"
+      "addc.cc.u32 %4, %4, %12;\n"
+      "addc.cc.u32 %5, %5, %13;\n"
+      "addc.cc.u32 %6, %6, %14;\n"
+      "addc.u32 %7, %7, %15;\n" "}"
+      : "+r"(T[0]), "+r"(T[1]), "+r"(T[2]), "+r"(T[3]), "+r"(T[4]), "+r"(T[5]), "+r"(T[6]), "+r"(T[7])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]), "r"(s));
+}
+template <>
+__device__ __forceinline__ void add_limbs32<10>(uint32_t (&T)[10], const uint32_t (&y)[10], uint32_t s) {
+  asm("{\n" ".reg .u32 c;\n"
+      "add.cc.u32 c, %20, %20;\n"
+      "addc.cc.u32 %0, %0, %10;\n"
+      "addc.cc.u32 %1, %1, %11;\n"
+      "addc.cc.u32 %2, %2, %12;\n"
+      "addc.cc.u32 %3, %3, %13;\n"
+      "addc.cc.u32 %4, %4, %14;\n"
+      "addc.cc.u32 %5, %5, %15;\n"
+      "addc.cc.u32 %6, %6, %16;\n"
+      "addc.cc.u32 %7, %7, %17;\n"
+      "addc.cc.u32 %8, %8, %18;\n"
+      "addc.u32 %9, %9, %19;\n" "}"
+      : "+r"(T[0]), "+r"(T[1]), "+r"(T[2]), "+r"(T[3]), "+r"(T[4]), "+r"(T[5]), "+r"(T[6]), "+r"(T[7]), "+r"(T[8]), "+r"(T[9])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]), "r"(y[8]), "r"(y[9]), "r"(s));
+}
+template <>
+__device__ __forceinline__ void add_limbs32<12>(uint32_t (&T)[12], const uint32_t (&y)[12], uint32_t s) {
+  asm("{\n" ".reg .u32 c;\n"
+      "add.cc.u32 c, %24, %24;\n"
+      "addc.cc.u32 %0, %0, %12;\n"
+      "addc.cc.u32 %1, %1, %13;\n"
+      "addc.cc.u32 %2, %2, %14;\n"
+      "addc.cc.u32 %3, %3, %15;\n"
+      "addc.cc.u32 %4, %4, %16;\n"
+      "addc.cc.u32 %5, %5, %17;\n"
+      "addc.cc.u32 %6, %6, %18;\n"
+      "addc.cc.u32 %7, %7, %19;\n"
+      "addc.cc.u32 %8, %8, %20;\n"
+      "addc.cc.u32 %9, %9, %21;\n"
+      "addc.cc.u32 %10, %10, %22;\n"
+      "addc.u32 %11, %11, %23;\n" "}"
+      : "+r"(T[0]), "+r"(T[1]), "+r"(T[2]), "+r"(T[3]), "+r"(T[4]), "+r"(T[5]), "+r"(T[6]), "+r"(T[7]), "+r"(T[8]), "+r"(T[9]), "+r"(T[10]), "+r"(T[11])
+      : "r"(y[0]), "r"(y[1]), "r"(y[2]), "r"(y[3]), "r"(y[4]), "r"(y[5]), "r"(y[6]), "r"(y[7]), "r"(y[8]), "r"(y[9]), "r"(y[10]), "r"(y[11]), "r"(s));
+}
+// Fixed-point values of the residue split: two's complement in NL 32-bit limbs.
+// T += trunc(x 2^F): the magnitude (53 bits, cut below weight 1) takes three limbs
+// from limb sh / 32 on; a barrel of selects over the bits of that limb index puts
+// them in place, and a negative word adds the complement of every limb plus one
+// (one carry chain either way, no branch on the sign).  The first word starts
+// from the bias H (kernel parameters), so the sum is T + H.
+template <int NL>
+__device__ __forceinline__ void add_word32(double x, int F, uint32_t (&T)[NL]) {
+  const uint32_t bh = (uint32_t)__double2hiint(x), bl = (uint32_t)__double2loint(x);
+  const int be = (int)((bh >> 20) & 0x7ffu);
+  int sh = max(be, 1) - 1075 + F;                  // weight of the last mantissa bit
+  uint64_t M = ((uint64_t)((bh & 0xFFFFFu) | (be ? 0x100000u : 0u)) << 32) | bl;
+  asm("shr.b64 %0, %0, %1;" : "+l"(M) : "r"(max(-sh, 0)));   // zero from 64 bits on
+  sh = max(sh, 0);
+  uint32_t s = (uint32_t)((int32_t)bh >> 31);
+  if (sh >= 32 * NL) {                             // only words the exponent does not cover
+    M = 0;                                         // (non-finite input, flagged elsewhere)
+    s = 0;
+    sh = 0;
+  }
+  const uint32_t lo = (uint32_t)M, hi = (uint32_t)(M >> 32);
+  const uint32_t v0 = (lo << (sh & 31)) ^ s, v1 = __funnelshift_l(lo, hi, sh) ^ s,
+                 v2 = __funnelshift_l(hi, 0u, sh) ^ s;
+  const bool b0 = sh & 32, b1 = sh & 64, b2 = sh & 128, b3 = sh & 256;
+  uint32_t w[4] = {b0 ? s : v0, b0 ? v0 : v1, b0 ? v1 : v2, b0 ? v2 : s};
+  uint32_t y[NL];
+  auto at1 = [&](int i) { return i >= 0 && i < 4 ? w[i] : s; };
+  auto at2 = [&](int i) { return i < 0 || i > 5 ? s : (b1 ? at1(i - 2) : at1(i)); };
+  uint32_t q[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) q[i] = at2(i);
+  uint32_t h[10];
+#pragma unroll
+  for (int i = 0; i < 10; ++i) {
+    const uint32_t plain = i < 6 ? q[i < 6 ? i : 0] : s, up = i >= 4 ? q[i >= 4 ? i - 4 : 0] : s;
+    h[i] = NL > 4 ? (b2 ? up : plain) : plain;
+  }
+#pragma unroll
+  for (int i = 0; i < NL; ++i) {
+    const uint32_t plain = i < 10 ? h[i < 10 ? i : 0] : s, up = i >= 8 ? h[i >= 8 ? i - 8 : 0] : s;
+    y[i] = NL > 8 ? (b3 ? up : plain) : plain;
+  }
+  add_limbs32<NL>(T, y, s);                        // carry in: one for a negative word
+}
+
+// T = S - H in [-2^(L-1), 2^(L-1)): every bit from L-1 up equals the sign.
+template <int NL>
+__device__ __forceinline__ bool in_range_bits(const uint32_t (&S)[NL], const uint32_t (&H)[NL],
+                                              int L) {
+  const int b = L - 1, lb = b >> 5, ob = b & 31;
+  uint32_t T[NL], v = 0, borrow = 0;
+#pragma unroll
+  for (int i = 0; i < NL; ++i) {
+    const uint64_t d = (uint64_t)S[i] - H[i] - borrow;
+    T[i] = (uint32_t)d;
+    borrow = (uint32_t)(d >> 32) & 1u;
+    if (i == lb) v = (uint32_t)((int32_t)T[i] >> ob);
+  }
+  bool ok = (v == 0u || v == 0xFFFFFFFFu) && lb < NL;
 #pragma unroll
   for (int i = 0; i < NL; ++i)
-    if (i == lb) v = (int64_t)T[i] >> ob;
-  bool ok = (v == 0 || v == -1) && lb < NL;
-#pragma unroll
-  for (int i = 0; i < NL; ++i)
-    if (i > lb) ok &= T[i] == (uint64_t)v;
+    if (i > lb) ok &= T[i] == v;
   return ok;
 }
 
@@ -156,9 +293,19 @@ __device__ __forceinline__ bool in_range_bits(const uint64_t (&T)[NL], int L) {
 // byte as low mantissa bits is 1024 + byte, so one byte permute and one packed
 // fp16 add of -1152 give two digits.  Every column gets byte - 128, the top
 // one too, whose digit is byte S-1 less 256 for a negative T + H: the
-// difference, +128 or -128, goes into column 63, whose constants are those of
-// column S-1 (S <= 48).  The other columns q >= S multiply zero constants and
-// may hold anything finite.
+// difference, +128 or -128, goes into the last column in use, Kc - 1 with
+// Kc = S + 1 rounded up to 16 (the K of the MMAs), whose constants are those of
+// column S-1.  The other columns q >= S multiply zero constants and may hold
+// anything finite.
+// Bound by the integer units (696 instructions a warp of entries before the last
+// trims, most of them selects, shifts and permutes; DRAM at half its rate), so the
+// words are placed by selects without branches, the sums reduced two moduli an
+// instruction (packed fp32), the range checked from the words' exponents, and only
+// columns in use written and multiplied.  Both operands with their exponents, us,
+// before / now: 4096^2 quad doubles 1,658 / 1,320, double doubles 1,226 / 882.
+// Measured and left out: 64-byte rows of A for a fourth CTA an SM (1,465), residues
+// stored from registers without the shared tile (1,671), words loaded two tiles
+// ahead (1,409), tiles of 4 r x 64 k (1,396 against 1,400 with 8 x 32 then).
 // TRANS = false: a tile is 256 consecutive k of one row r (slot = k); TRANS =
 // true (the operand stored K x R): 8 consecutive r x 32 consecutive k (slot =
 // 32 r + k), thread i reading r = i mod 8, k = i / 8, so that the loads along r
@@ -179,18 +326,54 @@ __host__ __device__ inline uint32_t residue_tmem_cols(int npad) {
 __host__ __device__ __forceinline__ uint32_t res_rho(uint32_t j) { return j ^ ((j >> 4) & 7u); }
 
 template <int MW>
-struct SplitEntry {      // one thread's entry of a tile: position and words
-  int64_t r, k;
+struct SplitEntry {      // one thread's entry of a tile: L - 2 - E and words
+  int F;
   bool valid;
   double x[MW];
 };
+template <int NL> struct BiasLimbs { uint32_t h[NL]; };   // H
+
+// Packed fp32 arithmetic (each element rounded as the scalar operation would).
+__device__ __forceinline__ uint64_t pk_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t pk_add(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t pk_make(uint32_t lo, uint32_t hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+  return d;
+}
+__device__ __forceinline__ void pk_split(uint64_t d, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(d));
+}
+
+// The balanced residues of two exactly represented float integers z (|z| < 2^22)
+// modulo the odd p_t and p_(t+1) (t even), in [-floor(p/2), floor(p/2)]: z - q p
+// with q the nearest integer to z / p.  fma(z, 1/p, 1.5 2^23) rounds the exact
+// product z fl(1/p) to an integer; that product differs from z / p by less than
+// |z| 2^-24 / p < 1 / (4p), while an integer z over an odd p lies at least
+// 1 / (2p) from any half integer, so q is the nearest integer to z / p itself.
+// Every step is exact (|q p| < 2^23).
+__device__ __forceinline__ uint64_t balanced_f2(uint64_t z, int t) {
+  const uint64_t rcp = *reinterpret_cast<const uint64_t *>(&kCrt.rcp[t]);
+  const uint64_t npf = *reinterpret_cast<const uint64_t *>(&kCrt.npf[t]);
+  const uint64_t q = pk_add(pk_fma(z, rcp, 0x4B4000004B400000ull), 0xCB400000CB400000ull);
+  return pk_fma(q, npf, z);
+}
 
 template <int MW, int NL, bool TRANS>
 __global__ void __launch_bounds__(kResTile, 3)
     residues_mma_kernel(const __grid_constant__ CUtensorMap omap, const double *__restrict__ X,
                         int64_t R, int64_t K, int64_t ld, int64_t ps, int L, int S, int nmod,
                         int npad, int64_t dld, const int *E, unsigned int *status,
-                        int32_t *redo, const int32_t *gate) {
+                        int32_t *redo, const int32_t *gate,
+                        const __grid_constant__ BiasLimbs<NL> H) {
   if (gate && *gate == 0) return;                  // the pass over every word is not needed
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sA = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);   // A_0, A_1
@@ -199,11 +382,12 @@ __global__ void __launch_bounds__(kResTile, 3)
   uint64_t *bar = (uint64_t *)(stage + (size_t)npad * 512);
   uint32_t *holder = (uint32_t *)(bar + 1);
   const int tid = threadIdx.x, warp = tid >> 5;
+  const int Kc = (S + 16) / 16 * 16;               // columns in use
   for (int idx = tid; idx < npad * 64; idx += kResTile) {
     const int t = idx >> 6, qc = idx & 63;
-    const int q = qc == 63 ? S - 1 : qc;       // column 63 repeats the top digit's
+    const int q = qc == Kc - 1 ? S - 1 : qc;   // the last column repeats the top digit's
     int c = 0;
-    if (t < nmod && (q < S || qc == 63)) {
+    if (t < nmod && q < S) {
       const uint32_t p = kCrt.p[t];
       uint32_t x = kCrt.pow16[t][q >> 1];
       if (q & 1) x = mod_u32(x * 256u, p, kCrt.m32[t]);
@@ -223,13 +407,15 @@ __global__ void __launch_bounds__(kResTile, 3)
   tc_fence_after();
   const uint32_t tmem = *holder;
   const uint32_t idesc = idesc_f16(128, npad);
-  const int64_t ktiles = TRANS ? (dld + 31) / 32 : (dld + 255) / 256;
-  const int64_t rtiles = TRANS ? (R + 7) / 8 : R;
+  // rows and columns fit in 31 bits (checked at the launch)
+  const uint32_t ktiles = (uint32_t)(TRANS ? (dld + 31) / 32 : (dld + 255) / 256);
+  const uint32_t rtiles = (uint32_t)(TRANS ? (R + 7) / 8 : R);
   // tile u = a * inner + b: (rt, kt) = (a, b) for rows (k contiguous), (b, a) for
   // the operand stored K x R, so that the CTAs running together read neighbouring
   // r of the same k rows (whole sectors); each CTA steps u by the grid size
-  const int64_t inner = TRANS ? rtiles : ktiles, outer = TRANS ? ktiles : rtiles;
-  const int64_t gq = gridDim.x / inner, gr = gridDim.x - gq * inner;
+  const uint32_t inner = TRANS ? rtiles : ktiles, outer = TRANS ? ktiles : rtiles;
+  const uint32_t gq = gridDim.x / inner, gr = gridDim.x - gq * inner;
+  const uint32_t uR = (uint32_t)R, uK = (uint32_t)K;
   // this thread's slot in the tile (the box is 256 k of one row, or 8 rows x 32
   // k), and the row of A_(slot & 1) that takes its digits
   const uint32_t slot = TRANS ? (uint32_t)((tid & 7) * 32 + (tid >> 3)) : (uint32_t)tid;
@@ -237,7 +423,7 @@ __global__ void __launch_bounds__(kResTile, 3)
   const uint32_t rowA = res_rho(slot >> 1);
   volatile int abort_flag = 0;
 
-  auto step = [&](int64_t &a, int64_t &b) {
+  auto step = [&](uint32_t &a, uint32_t &b) {
     a += gq;
     b += gr;
     if (b >= inner) {
@@ -245,68 +431,75 @@ __global__ void __launch_bounds__(kResTile, 3)
       ++a;
     }
   };
-  auto fetch = [&](int64_t ta, int64_t tb, SplitEntry<MW> &e) {
-    e.valid = false;
-    e.r = e.k = 0;
-    if (ta < outer) {
-      const int64_t rt = TRANS ? tb : ta, kt = TRANS ? ta : tb;
-      e.r = TRANS ? rt * 8 + (tid & 7) : rt;
-      e.k = TRANS ? kt * 32 + (tid >> 3) : kt * 256 + tid;
-      e.valid = e.r < R && e.k < dld;
-    }
-    const bool in = e.valid && e.k < K;
+  auto fetch = [&](uint32_t ta, uint32_t tb, SplitEntry<MW> &e) {
+    const uint32_t rt = TRANS ? tb : ta, kt = TRANS ? ta : tb;
+    const uint32_t r = TRANS ? rt * 8 + (tid & 7) : rt;
+    const uint32_t k = TRANS ? kt * 32 + (tid >> 3) : kt * 256 + tid;
+    e.valid = ta < outer && r < uR && k < uK;      // entries from K up are zeros
+    e.F = e.valid ? L - 2 - E[r] : 0;
+    const double *p = X + (TRANS ? (int64_t)k * ld + r : (int64_t)r * ld + k);
 #pragma unroll
-    for (int j = 0; j < MW; ++j)
-      e.x[j] = in ? (TRANS ? X[j * ps + e.k * ld + e.r] : X[j * ps + e.r * ld + e.k]) : 0.0;
+    for (int j = 0; j < MW; ++j) e.x[j] = e.valid ? p[j * ps] : 0.0;
   };
 
   SplitEntry<MW> ec, en;
   uint32_t ph = 0;
   bool ok = true;
-  int64_t ca = blockIdx.x / inner, cb = blockIdx.x - (blockIdx.x / inner) * inner;
+  uint32_t ca = blockIdx.x / inner, cb = blockIdx.x - (blockIdx.x / inner) * inner;
   fetch(ca, cb, ec);
   for (; ca < outer; step(ca, cb)) {
-    // digits of the entry into row tid of A
+    // digits of the entry into its row of A
     {
-      uint64_t T[NL];
-      fixed_point<MW, NL>(ec.x, ec.valid ? L - 2 - E[ec.r] : 0, T);
-      const bool in = in_range_bits<NL>(T, L);
-      if (redo) {
-        // exponents from the leading words: they hold for this entry when its
-        // leading word is normal and no later word has a larger exponent field, or
-        // when every word is zero; anything else (and a value out of range) sends
-        // the operand through the pass over every word
-        const uint32_t e0 = (uint32_t)(__double_as_longlong(ec.x[0]) >> 52) & 0x7ffu;
-        bool lead = e0 != 0x7ffu;
-        bool rest = false;                         // a later word is nonzero
+      uint32_t T[NL];                              // T + H
 #pragma unroll
-        for (int j = 1; j < MW; ++j) {
-          const uint64_t b = (uint64_t)__double_as_longlong(ec.x[j]);
-          const uint32_t ej = (uint32_t)(b >> 52) & 0x7ffu;
-          lead &= ej <= e0 && ej != 0x7ffu;
-          rest |= (b << 1) != 0;
-        }
-        if (e0 == 0) lead = !rest;                 // zero or subnormal, the only nonzero word
-        if (ec.valid && !(lead && in)) atomicExch(redo, 1);
-      } else if (ec.valid && !in) {
-        raise_status(status, MW_ERANGE);
+      for (int i = 0; i < NL; ++i) T[i] = H.h[i];
+      // later words two binary orders below the leading one: |T| < 2^(L-1), and the
+      // leading word holds the exponent (so zero entries take the exact check)
+      const int e0 = (int)((uint32_t)__double2hiint(ec.x[0]) >> 20) & 0x7ff;
+      bool plain = e0 != 0x7ff;
+#pragma unroll
+      for (int j = 0; j < MW; ++j) {
+        if (j) plain &= (int)(((uint32_t)__double2hiint(ec.x[j]) >> 20) & 0x7ffu) + 2 <= e0;
+        add_word32<NL>(ec.x[j], ec.F, T);
       }
-      const bool neg = add_bias_w8<NL>(T, S);
+      if (!plain && ec.valid) {
+        const bool in = in_range_bits<NL>(T, H.h, L);
+        if (redo) {
+          // exponents from the leading words: they hold for this entry when its
+          // leading word is normal and no later word has a larger exponent field, or
+          // when every word is zero; anything else (and a value out of range) sends
+          // the operand through the pass over every word
+          bool lead = e0 != 0x7ff;
+          bool rest = false;                       // a later word is nonzero
+#pragma unroll
+          for (int j = 1; j < MW; ++j) {
+            const uint64_t b = (uint64_t)__double_as_longlong(ec.x[j]);
+            const int ej = (int)(b >> 52) & 0x7ff;
+            lead &= ej <= e0 && ej != 0x7ff;
+            rest |= (b << 1) != 0;
+          }
+          if (e0 == 0) lead = !rest;               // zero or subnormal, the only nonzero word
+          if (!(lead && in)) atomicExch(redo, 1);
+        } else if (!in) {
+          raise_status(status, MW_ERANGE);
+        }
+      }
+      const uint32_t last = (int32_t)T[NL - 1] < 0 ? 0xD8000000u : 0x58000000u;   // -128, 128
 #pragma unroll
       for (int c = 0; c < 8; ++c) {               // 16-byte chunk c: digits 8c .. 8c+7
+        if (8 * c >= Kc) break;
         uint32_t w[4] = {0u, 0u, 0u, 0u};
-        if (c < NL) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t word = (uint32_t)(T[c < NL ? c : 0] >> (32 * h));
+        for (int h = 0; h < 2; ++h)
+          if (2 * c + h < NL) {
+            const uint32_t word = T[2 * c + h < NL ? 2 * c + h : 0];
             uint32_t lo, hi;
             asm("prmt.b32 %0, %1, %2, 0x5140;" : "=r"(lo) : "r"(word), "r"(0x64646464u));
             asm("prmt.b32 %0, %1, %2, 0x7362;" : "=r"(hi) : "r"(word), "r"(0x64646464u));
             asm("add.rn.f16x2 %0, %1, %2;" : "=r"(w[2 * h]) : "r"(lo), "r"(0xE480E480u));
             asm("add.rn.f16x2 %0, %1, %2;" : "=r"(w[2 * h + 1]) : "r"(hi), "r"(0xE480E480u));
           }
-        }
-        if (c == 7) w[3] = neg ? 0xD8000000u : 0x58000000u;   // column 63: -128 / +128 in fp16
+        if (8 * c + 8 == Kc) w[3] = (w[3] & 0xFFFFu) | last;   // column Kc - 1
         *reinterpret_cast<uint4 *>(arow + sw128_offset(rowA, 8 * c)) = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
@@ -317,15 +510,14 @@ __global__ void __launch_bounds__(kResTile, 3)
       tc_fence_after();
       const uint64_t a0 = sw128_desc(smem_u32(sA)), a1 = sw128_desc(smem_u32(sA + kHalfBytes));
       const uint64_t bd = sw128_desc(smem_u32(sB));
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) tc_mma(tmem, a0 + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : 0u);
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
+      for (int kk = 0; 16 * kk < Kc; ++kk)
+        tc_mma(tmem, a0 + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : 0u);
+      for (int kk = 0; 16 * kk < Kc; ++kk)
         tc_mma(tmem + npad, a1 + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : 0u);
       tc_commit(&bar[0]);
     }
     {
-      int64_t na = ca, nb = cb;
+      uint32_t na = ca, nb = cb;
       step(na, nb);
       fetch(na, nb, en);                           // the next tile's words load meanwhile
     }
@@ -351,13 +543,15 @@ __global__ void __launch_bounds__(kResTile, 3)
           tc_ld16(ta + npad + t0, vo);
           tc_wait_ld();
 #pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            if (t0 + u >= nmod) break;
-            const float re = balanced_f(__uint_as_float(ve[u]), 32 * h + 16 * HF + u);
-            const float ro = balanced_f(__uint_as_float(vo[u]), 32 * h + 16 * HF + u);
+          for (int u = 0; u < 16; u += 2) {       // columns from nmod on: zeros, never stored
+            float e0, e1, o0, o1;
+            pk_split(balanced_f2(pk_make(ve[u], ve[u + 1]), 32 * h + 16 * HF + u), e0, e1);
+            pk_split(balanced_f2(pk_make(vo[u], vo[u + 1]), 32 * h + 16 * HF + u), o0, o1);
             uint32_t pr;
-            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pr) : "f"(ro), "f"(re));
+            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pr) : "f"(o0), "f"(e0));
             dst[(size_t)(t0 + u) * 128] = pr;
+            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(pr) : "f"(o1), "f"(e1));
+            dst[(size_t)(t0 + u + 1) * 128] = pr;
           }
         }
       };
@@ -389,7 +583,7 @@ template <int MW, int NL>
 int launch_residues_t(const SplitArgs &a, cudaStream_t s) {
   const int S = (a.S + 7) / 8;                     // base-256 digits of an L-bit T
   const int npad = (a.nmod + 15) / 16 * 16;
-  if (S > 8 * NL || S > 48 || NL > 6 || npad > 96)
+  if (S > 4 * NL || S > 48 || npad > 96)
     return fail(MW_EUNSUPPORTED, "residue split: %d digits, %d moduli", S, a.nmod);
   if (a.digit_ld % 8 || a.R > 0x7fffffffLL || a.digit_ld > 0x7fffffffLL)
     return fail(MW_EUNSUPPORTED, "residue split: planes of %lld x %lld", (long long)a.R,
@@ -429,17 +623,29 @@ int launch_residues_t(const SplitArgs &a, cudaStream_t s) {
   const int64_t ktiles = a.trans ? (a.digit_ld + 31) / 32 : (a.digit_ld + 255) / 256;
   const int64_t ntiles = (a.trans ? (a.R + 7) / 8 : a.R) * ktiles;
   const unsigned grid = (unsigned)std::min<int64_t>(ntiles, (int64_t)per_sm * nsm);
+  BiasLimbs<NL> H;                                 // 128 in every byte below the top digit
+  for (int i = 0; i < NL; ++i) {
+    const int nb = std::min(std::max(S - 1 - 4 * i, 0), 4);
+    H.h[i] = (uint32_t)(0x80808080ull & ((1ull << (8 * nb)) - 1));
+  }
   kern<<<grid, kResTile, smem, s>>>(map, a.X, a.R, a.K, a.ld, a.plane_stride, a.S, S, a.nmod,
-                                    npad, a.digit_ld, a.exps, status_ptr(), a.redo, a.gate);
+                                    npad, a.digit_ld, a.exps, status_ptr(), a.redo, a.gate, H);
   return cuda_fail(cudaGetLastError(), "residue split launch");
 }
 
 template <int MW>
 int launch_residues_nl(const SplitArgs &a, cudaStream_t s) {
   const int bits = a.S + 3;    // |T| < m 2^(L-2) < 2^(L+1), one sign bit
-  if (bits <= 128) return launch_residues_t<MW, 2>(a, s);
-  if (bits <= 256) return launch_residues_t<MW, 4>(a, s);
-  if (bits <= 384) return launch_residues_t<MW, 6>(a, s);
+  if constexpr (MW == 2) {     // 104 bits and the spread
+    if (bits <= 128) return launch_residues_t<MW, 4>(a, s);
+    if (bits <= 160) return launch_residues_t<MW, 5>(a, s);
+    if (bits <= 192) return launch_residues_t<MW, 6>(a, s);
+  } else {                     // 208 bits and the spread
+    if (bits <= 224) return launch_residues_t<MW, 7>(a, s);
+  }
+  if (bits <= 256) return launch_residues_t<MW, 8>(a, s);
+  if (bits <= 320) return launch_residues_t<MW, 10>(a, s);
+  if (bits <= 384) return launch_residues_t<MW, 12>(a, s);
   return fail(MW_EUNSUPPORTED, "residue form: %d fixed-point bits (at most 381)", a.S);
 }
 
