@@ -205,46 +205,45 @@ MW_HD bool cut_column(const double (&x)[MW], int F, int S, uint32_t *col, int st
 template <int MW, int NL32, class Store>
 MW_HD void round_column(const uint32_t (&U)[NL32], uint32_t *col, int stride, int ex,
                         Store store) {
-  int lw = -1;
-  uint32_t lv = 0;
+  int lw = 0;
+  uint32_t lv = U[0];
 #pragma unroll
-  for (int i = NL32 - 1; i >= 0; --i) {
-    col[i * stride] = U[i];
-    if (U[i] != 0) {
-      lw = i;
-      lv = U[i];
-    }
+  for (int i = 0; i < NL32; ++i) col[i * stride] = U[i];
+  if (lv == 0) {                                    // rare: the last limb is zero
+    lw = -1;
+#pragma unroll
+    for (int i = NL32 - 1; i >= 1; --i)
+      if (U[i] != 0) {
+        lw = i;
+        lv = U[i];
+      }
   }
   int k = 0;
   if (lw >= 0) {
     const int ell = 32 * lw + col_ctz(lv);
     const uint32_t inv_l = ~((2u << (ell & 31)) - 1u);    // bits above l in limb lw
-    bool flip = (int32_t)U[NL32 - 1] < 0;                 // reading: inverted above l
-    bool neg = flip;
+    uint32_t flip = (uint32_t)((int32_t)U[NL32 - 1] >> 31);   // all ones: inverted above l
+    uint32_t neg = flip & 0x80000000u;
     int cutp = 32 * NL32;                                 // bits at and above are cleared
 #pragma unroll 1
     for (; k < MW && ell < cutp; ++k) {
-      const int Lc = cutp >> 5;
-      const uint32_t cm = (1u << (cutp & 31)) - 1u;
-      auto limb = [&](int L) -> uint32_t {
+      auto limb = [&](int L) -> uint32_t {                // below the cut
         if (L < 0) return 0u;
-        uint32_t v = col[L * stride];
-        if (flip) v ^= L > lw ? 0xFFFFFFFFu : (L == lw ? inv_l : 0u);
-        return L < Lc ? v : (L == Lc ? (v & cm) : 0u);
+        return col[L * stride] ^ (flip & (L > lw ? 0xFFFFFFFFu : (L == lw ? inv_l : 0u)));
       };
       int h = (cutp - 1) >> 5;
       uint32_t a = limb(h);
+      if (cutp & 31) a &= (1u << (cutp & 31)) - 1u;
       while (a == 0 && h > lw) a = limb(--h);           // bit l is set: ends at lw at the latest
       const uint32_t b = limb(h - 1), c = limb(h - 2);
       const bool below = ell < 32 * (h - 2);
       const int lz = col_clz(a);
-      const uint64_t ab = ((uint64_t)a << 32) | b;
-      const uint64_t top = lz ? (ab << lz) | (c >> (32 - lz)) : ab;
-      const uint32_t c_low = c << lz;                     // bits of c below the window
-      uint64_t mant = top >> 11;
-      const uint32_t rbit = (uint32_t)(top >> 10) & 1u;
-      const bool sticky = ((top & 0x3FF) | c_low) != 0 || below;
-      const uint32_t up = rbit & (uint32_t)(sticky | (mant & 1));
+      // the 64 bits from the top one on, then the bits of c below them
+      const uint32_t t1 = col_fshl(b, a, lz), t0 = col_fshl(c, b, lz), c_low = c << lz;
+      uint64_t mant = ((uint64_t)(t1 >> 11) << 32) | col_fshr(t0, t1, 11);
+      const uint32_t rbit = (t0 >> 10) & 1u;
+      const bool sticky = ((t0 & 0x3FFu) | c_low) != 0 || below;
+      const uint32_t up = rbit & (uint32_t)(sticky | (t0 >> 11 & 1u));
       mant += up;
       const int cut = 32 * h - 21 - lz;                   // weight of the mantissa's last bit
       const int e = ex + cut;
@@ -254,10 +253,10 @@ MW_HD void round_column(const uint32_t (&U)[NL32], uint32_t *col, int stride, in
         mag = col_double(((uint64_t)bexp << 52) + (mant - (1ull << 52)));
       else
         mag = scalbn((double)mant, e);
-      store(k, neg ? -mag : mag);
+      store(k, col_double(col_bits(mag) ^ ((uint64_t)neg << 32)));
       if (up) {
-        flip = !flip;
-        neg = !neg;
+        flip = ~flip;
+        neg ^= 0x80000000u;
       }
       cutp = cut;
     }
