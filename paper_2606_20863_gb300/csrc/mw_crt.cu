@@ -659,58 +659,80 @@ int launch_residues_nl(const SplitArgs &a, cudaStream_t s) {
 // per tile of 128 outputs (A: 128 x D residues, B: D x 4 NL bytes), |z_n| <= 96
 // 2^15 < 2^22.  The accumulators start at 1.5 2^23 (written into tensor memory
 // before each product), so every partial sum is an integer in [2^23, 2^24) (exact)
-// and the accumulator's bits are 0x4B400000 + z_n.  Horner joins them into
-// 32-bit limbs, k comes from the limbs top-2..top of X' (|X'| < D 2^8 P), and
-// X = X' + |k| (P or 2^(32 NL) - P) mod 2^(32 NL) is rounded greedily into m words.
+// and the accumulator's bits are 0x4B400000 + z_n.
+// k comes first, from the float sum of the eight highest z_n 2^(8n) / P: the
+// others are below 2^(22 + 8 (4 top - 9) + 1) < 2^-7 P and the rounding of sums
+// below 2^16 errs by less than 2^-5, where |X| < P/8 leaves 3/8.  Then one pass
+// gives the limbs of X: limb l adds z_4l .. z_4l+3 at their bytes, the bias's
+// complement c_l and -k times p_l (P in balanced 32-bit limbs), all multiply-adds
+// of 32 x 32 -> 64 bits, and the carry of limb l - 1.  X is rounded greedily into
+// m words.
+//
+// The residues of a tile arrive by TMA as rows t of 64 outputs (two boxes, 128-byte
+// swizzle), which is the layout of an A operand with M contiguous, so the MMA reads
+// them as they are.  One accumulator: a tile's product is issued when the previous
+// tile's sums have been read and runs while that tile is rounded; two buffers of
+// residues, the one just multiplied serving as the limb columns of the rounding
+// before its next load.  Bound by integer issue and latency: the kernel before this
+// (residues transposed through registers into a K-major A, two accumulators, X'
+// stored and read again for k) took 1,067 us for 4096^2 quad doubles, 781 us for
+// double doubles and 94 us for 777 x 1300 quad doubles; now 706, 527 and 72 us (with
+// the faster round_column).
 struct CrtFuse {
   int D, top;                                      // moduli; limbs of X' below its sign
-  float c64, c32;                                  // 2^(32(top - 1)) / P, 2^(32(top - 2)) / P
+  uint32_t byte1, byte2, byte3;                    // 2^8, 2^16, 2^24
+  float cz[8];                                     // 2^(8 (4 top - 8 + i)) / P
   int8_t qb[kCrtMaxModuli][4 * kCrtMaxLimbs];      // balanced bytes of Q'_t
-  uint32_t P[kCrtMaxLimbs], nP[kCrtMaxLimbs];      // P and 2^(32 NL) - P
+  int32_t P[kCrtMaxLimbs];                         // balanced limbs of P
+  uint32_t bias[kCrtMaxLimbs];                     // -sum_n 0x4B400000 2^(8n) mod 2^(32 NL)
 };
 
 template <int NL>
 struct FuseShape {
   static constexpr int NB = 4 * NL;                // byte positions: N of the MMA
-  static constexpr uint32_t TCOLS = 2 * NB <= 128 ? 128u : 256u;   // two accumulators
+  static constexpr uint32_t TCOLS = NB <= 32 ? 32u : NB <= 64 ? 64u : 128u;
 };
 
-// Bytes of shared memory the reconstruction kernel uses for D moduli and NL limbs
-// (with the rounding's limb columns in shared memory unless LCOL).
-inline size_t fuse_smem(int D, int NL, bool lcol) {
-  const int D8 = (D + 7) & ~7, KM = (D8 + 15) & ~15, kc = (KM + 63) / 64;
-  return 1024 + (size_t)256 * D8 + (size_t)kc * 16384 + (size_t)kc * 4 * NL * 128 +
-         (lcol ? 0 : (size_t)(NL + 1) * 512) + 32;
+// Bytes of shared memory the reconstruction kernel uses for D moduli and NL limbs.
+inline size_t fuse_smem(int D, int NL) {
+  const int KM = (D + 15) & ~15, kc = (KM + 63) / 64;
+  return 1024 + (size_t)2 * 256 * KM + (size_t)kc * 4 * NL * 128 + 48;
 }
 
-template <int MW, int NL, bool LCOL>
-__global__ void __launch_bounds__(128, 2)
+// acc + a b with a 64-bit sum, one instruction.
+__device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t b, uint64_t acc) {
+  uint64_t d;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(acc));
+  return d;
+}
+__device__ __forceinline__ uint64_t mad_wide_s(int32_t a, int32_t b, uint64_t acc) {
+  uint64_t d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(acc));
+  return d;
+}
+
+template <int MW, int NL>
+__global__ void __launch_bounds__(128, NL <= 16 ? 5 : 4)
     crt_fuse_kernel(const __grid_constant__ CUtensorMap map, const int32_t *eA, const int32_t *eB,
                     int64_t M, int64_t N, int ex0, double *C, int64_t ldc, int64_t psc,
                     unsigned int *status, const __grid_constant__ CrtFuse F) {
   constexpr int NB = FuseShape<NL>::NB;
   constexpr uint32_t TCOLS = FuseShape<NL>::TCOLS;
-  const int D = F.D, D8 = (D + 7) & ~7;
-  const int KM = (D8 + 15) & ~15, kc = (KM + 63) / 64;
+  const int D = F.D, KM = (D + 15) & ~15, kc = (KM + 63) / 64;
   extern __shared__ uint8_t smem_raw[];
-  // residues of a tile (128 outputs of one row) as TMA leaves them (two halves of
-  // 64, D8 rows of 128 B, swizzled), the MMA's A (128 rows, K-major) and B (NB
-  // rows), then (unless LCOL: each thread's local memory, when shared memory would
-  // hold fewer CTAs than the tensor memory) the limbs the rounding reads by index
+  // two buffers of residues (two halves of 64 outputs, KM rows of 128 B each), then
+  // the MMA's B (NB rows, K-major)
   uint8_t *stage = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t *sA = stage + 256 * D8;
-  uint8_t *sB = sA + kc * 16384;
-  uint32_t *colsm = (uint32_t *)(sB + kc * NB * 128);        // [NL + 1][128] unless LCOL
-  uint64_t *bar = (uint64_t *)(colsm + (LCOL ? 0 : (NL + 1) * 128));   // residues, accumulators
+  const uint32_t stage_bytes = 256u * KM;
+  uint8_t *sB = stage + 2 * stage_bytes;
+  uint64_t *bar = (uint64_t *)(sB + kc * NB * 128);          // residues [2], product
   uint32_t *holder = (uint32_t *)(bar + 3);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5;
   for (int idx = tid; idx < kc * 64 * NB; idx += 128) {
     const int t = idx / NB, n = idx - t * NB;
     const uint16_t v = t < D ? small_int_bf16(F.qb[t][n]) : (uint16_t)0;
     *reinterpret_cast<uint16_t *>(sB + (t >> 6) * (NB * 128) + sw128_offset(n, t & 63)) = v;
   }
-  for (int t = D8; t < kc * 64; ++t)               // row tid of A past the residues
-    *reinterpret_cast<uint16_t *>(sA + (t >> 6) * 16384 + sw128_offset(tid, t & 63)) = 0;
   if (tid == 0) {
     for (int b = 0; b < 3; ++b) mbar_init(&bar[b], 1);
     fence_barrier_init();
@@ -721,159 +743,117 @@ __global__ void __launch_bounds__(128, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *holder;
-  // the bias 1.5 2^23 into this warp's lanes of both accumulators
-  auto bias_fill = [&](int s) {
-    const uint32_t ta = tmem + s * NB + ((uint32_t)(warp * 32) << 16);
+  const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
+  auto bias_fill = [&]() {                         // 1.5 2^23 into this warp's lanes
 #pragma unroll
     for (int h = 0; h < (NB + 31) / 32; ++h) {
       if (32 * h + 32 <= NB) tc_fill32(ta + 32 * h, 0x4B400000u);
       else tc_fill16(ta + 32 * h, 0x4B400000u);
     }
   };
-  bias_fill(0);
-  bias_fill(1);
+  bias_fill();
   tc_wait_st();
   tc_fence_before();
   __syncthreads();
-  const uint32_t idesc = idesc_bf16(128, NB);
+  // A with M contiguous (bit 15): 64-output groups `half` bytes apart, 8 moduli 1024
+  const uint32_t idesc = idesc_bf16(128, NB) | (1u << 15);
+  const uint32_t half = 128u * KM;
   const int64_t jtiles = (N + 127) / 128, ntiles = jtiles * M;   // a tile: 128 j of one row i
-  const uint32_t stage_bytes = 256u * D8;
   volatile int abort_flag = 0;
 
-  auto issue = [&](int64_t tile) {                // one thread: the tile's residues
+  auto load = [&](int64_t tile, int s) {           // one thread: the tile's residues
     const int64_t i = tile / jtiles, j0 = (tile - i * jtiles) * 128;
-    mbar_arrive_expect_tx(&bar[0], stage_bytes);
-    tma_load_3d(smem_u32(stage), &map, (int)j0, (int)i, 0, smem_u32(&bar[0]));
-    tma_load_3d(smem_u32(stage + 128 * D8), &map, (int)j0 + 64, (int)i, 0, smem_u32(&bar[0]));
+    uint8_t *p = stage + s * stage_bytes;
+    mbar_arrive_expect_tx(&bar[s], stage_bytes);
+    tma_load_3d(smem_u32(p), &map, (int)j0, (int)i, 0, smem_u32(&bar[s]));
+    tma_load_3d(smem_u32(p + half), &map, (int)j0 + 64, (int)i, 0, smem_u32(&bar[s]));
   };
-  // staged residues (rows t, outputs along the row) into A (rows = outputs):
-  // warp w moves outputs 32w..32w+31, eight moduli per step
-  auto transpose = [&]() {
-    const int c = 4 * warp + (lane >> 3), rho = lane & 7;
-    const uint32_t src = smem_u32(stage) + (c >> 3) * (128 * D8) + rho * 128 + (((c & 7) ^ rho) << 4);
-    const uint32_t dst = smem_u32(sA) + (8 * c + rho) * 128;
-    for (int tau = 0; tau < D8 / 8; ++tau) {
-      uint32_t r[4];
-      ldsm_x4_trans(src + tau * 1024, r);
-      stsm_x4(dst + (tau >> 3) * 16384 + (((tau & 7) ^ rho) << 4), r);
-    }
-  };
-  uint32_t fph = 0, mph[2] = {0u, 0u};
-  // X' from the accumulator of `tile`, k, X, greedy words
-  auto drain = [&](int64_t tile, int s) -> bool {
-    if (!__syncthreads_and(mbar_wait(&bar[1 + s], mph[s], status, &abort_flag))) return false;
-    mph[s] ^= 1;
+  auto product = [&](int s) {                      // one thread: onto the bias
     tc_fence_after();
-    const uint32_t ta = tmem + s * NB + ((uint32_t)(warp * 32) << 16);
-    constexpr uint64_t K0 = 0x4B400000ull * 0x01010101ull;   // the bias in a limb's four bytes
-    uint32_t U[NL];
-    int64_t rc = 0;
-#pragma unroll
-    for (int h = 0; h < (NB + 31) / 32; ++h) {
-      uint32_t z[32];
-      if (32 * h + 32 <= NB) tc_ld32(ta + 32 * h, z);
-      else tc_ld16(ta + 32 * h, z);
-      tc_wait_ld();
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (32 * h + 4 * q >= NB) break;
-        const int64_t acc = rc - (int64_t)K0 + (int64_t)z[4 * q] + ((int64_t)z[4 * q + 1] << 8) +
-                            ((int64_t)z[4 * q + 2] << 16) + ((int64_t)z[4 * q + 3] << 24);
-        U[8 * h + q] = (uint32_t)acc;
-        rc = acc >> 32;
-      }
+    for (int cc = 0; cc < kc; ++cc) {
+      const uint64_t ad = mn128_desc(smem_u32(stage + s * stage_bytes) + cc * 8192, half);
+      const uint64_t bd = sw128_desc(smem_u32(sB + cc * NB * 128));
+      for (int kk = 0; kk < 4 && 64 * cc + 16 * kk < KM; ++kk)
+        tc_mma(tmem, ad + 128 * kk, bd + 2 * kk, idesc, 1u);
     }
-    bias_fill(s);                                  // for the accumulator's next product
-    tc_wait_st();
-    tc_fence_before();
-    const int64_t i = tile / jtiles, j = (tile - i * jtiles) * 128 + tid;
-    uint32_t lcol[LCOL ? NL + 1 : 1];              // read by index: local memory
-    uint32_t *col = LCOL ? lcol : colsm + tid;
-    constexpr int cs = LCOL ? 1 : 128;
-#pragma unroll
-    for (int l = 0; l < NL; ++l) col[l * cs] = U[l];
-    col[NL * cs] = (uint32_t)rc;
-    const int top = F.top;
-    const uint64_t hi = ((uint64_t)col[top * cs] << 32) | col[(top - 1) * cs];
-    const float kf = fmaf((float)(int64_t)hi, F.c64, (float)col[(top - 2) * cs] * F.c32);
-    const int k = (int)(__float_as_uint(kf + 12582912.0f) - 0x4B400000u);
-    const bool pos = k > 0;
-    const uint32_t ak = (uint32_t)(pos ? k : -k);
-    uint64_t cy = 0;
-#pragma unroll
-    for (int l = 0; l < NL; ++l) {
-      const uint64_t v = (uint64_t)ak * (pos ? F.nP[l] : F.P[l]) + U[l] + cy;
-      U[l] = (uint32_t)v;
-      cy = v >> 32;
-    }
-    if (j < N) {
-      double *c = C + i * ldc + j;
-      round_column<MW, NL>(U, col, cs, eA[i] + eB[j] + ex0,
-                           [&](int wd, double v) { c[wd * psc] = v; });
-    }
-    return true;
+    tc_commit(&bar[2]);
   };
 
-  // the next tile's residues load while this tile is moved and the previous
-  // tile drains; its product runs during that drain
-  int64_t cur = blockIdx.x, prev = -1;
-  int slot = 0;
-  bool ok = true, tma_out = false;
-  uint32_t mma_out = 0;                            // accumulators with a product in flight
-  if (tid == 0 && cur < ntiles) {
-    issue(cur);
-    tma_out = true;
+  // tile q of this CTA: residues in buffer q & 1 (their phase (q >> 1) & 1), product
+  // phase q & 1
+  bool ok = true, load_out = false, product_out = false;   // in flight (thread 0)
+  uint32_t q = 0;
+  if (tid == 0 && blockIdx.x < ntiles) {
+    load(blockIdx.x, 0);
+    load_out = true;
   }
-  while (ok && (cur < ntiles || prev >= 0)) {
-    const bool have = cur < ntiles;
-    if (have) {
-      ok = __syncthreads_and(mbar_wait(&bar[0], fph, status, &abort_flag));
-      if (!ok) break;
-      fph ^= 1;
-      tma_out = false;
-      // the previous product has read A before A is rewritten
-      if (prev >= 0 && !__syncthreads_and(mbar_wait(&bar[1 + (slot ^ 1)], mph[slot ^ 1], status,
-                                                    &abort_flag))) {
-        ok = false;
-        break;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++q) {
+    const int s = q & 1;
+    if (tid == 0) {
+      ok = mbar_wait(&bar[s], (q >> 1) & 1, status, &abort_flag);
+      if (ok) {
+        load_out = false;
+        product(s);
+        product_out = true;
       }
-      transpose();
-      fence_proxy_async_smem();
-      __syncthreads();
-      if (tid == 0) {
-        if (cur + gridDim.x < ntiles) {
-          issue(cur + gridDim.x);
-          tma_out = true;
-        }
-        tc_fence_after();
-        const uint32_t d = tmem + slot * NB;
-        for (int cc = 0; cc < kc; ++cc) {
-          const uint64_t ad = sw128_desc(smem_u32(sA + cc * 16384));
-          const uint64_t bd = sw128_desc(smem_u32(sB + cc * NB * 128));
-          for (int kk = 0; kk < 4 && 64 * cc + 16 * kk < KM; ++kk)
-            tc_mma(d, ad + 2 * kk, bd + 2 * kk, idesc, 1u);   // onto the bias
-        }
-        tc_commit(&bar[1 + slot]);
+    }
+    if (ok) ok = mbar_wait(&bar[2], q & 1, status, &abort_flag);
+    if (ok) product_out = false;
+    tc_fence_after();
+    // k
+    uint32_t zt[8];
+    tc_ld8(ta + 4 * F.top - 8, zt);
+    tc_wait_ld();
+    float kf = 0.0f;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) kf = fmaf(__uint_as_float(zt[n]) - 12582912.0f, F.cz[n], kf);
+    const int nk = (int)(0x4B400000u - __float_as_uint(kf + 12582912.0f));
+    // X
+    uint32_t U[NL];
+    uint64_t acc = 0;
+#pragma unroll
+    for (int h = 0; h < NB / 16; ++h) {
+      uint32_t z[16];
+      tc_ld16(ta + 16 * h, z);
+      tc_wait_ld();
+#pragma unroll
+      for (int n = 0; n < 4; ++n) {
+        const int l = 4 * h + n;
+        acc = mad_wide_s(nk, F.P[l], acc);
+        acc += (uint64_t)z[4 * n] + F.bias[l];
+        acc = mad_wide(z[4 * n + 1], F.byte1, acc);
+        acc = mad_wide(z[4 * n + 2], F.byte2, acc);
+        acc = mad_wide(z[4 * n + 3], F.byte3, acc);
+        U[l] = (uint32_t)acc;
+        acc = (uint64_t)((int64_t)acc >> 32);
       }
-      mma_out |= 1u << slot;
     }
-    if (prev >= 0) {
-      ok = drain(prev, slot ^ 1);
-      if (!ok) break;
-      mma_out &= ~(1u << (slot ^ 1));
+    bias_fill();                                   // for the next tile's product
+    tc_wait_st();
+    tc_fence_before();
+    fence_proxy_async_smem();                      // the previous tile's limb columns
+    ok = __syncthreads_and(ok);
+    if (!ok) break;
+    if (tid == 0 && tile + gridDim.x < ntiles) {   // into the buffer those columns used
+      load(tile + gridDim.x, s ^ 1);
+      load_out = true;
     }
-    prev = have ? cur : -1;
-    if (have) cur += gridDim.x;
-    slot ^= 1;
+    const int64_t i = tile / jtiles, j = (tile - i * jtiles) * 128 + tid;
+    if (j < N) {
+      uint32_t *col = reinterpret_cast<uint32_t *>(stage + s * stage_bytes) + tid;
+      double *c = C + i * ldc + j;
+      round_column<MW, NL>(U, col, 128, eA[i] + eB[j] + ex0,
+                           [&](int wd, double v) { c[wd * psc] = v; });
+    }
   }
-  // after a wait that gave up: let the copies and products in flight finish
+  // after a wait that gave up: let the copies and the product in flight finish
   // (bounded) before the tensor memory is released
   if (!ok && tid == 0) {
     volatile int never = 0;
-    if (tma_out) mbar_wait(&bar[0], fph, status, &never);
-    for (int s = 0; s < 2; ++s)
-      if (mma_out & (1u << s)) mbar_wait(&bar[1 + s], mph[s], status, &never);
+    if (load_out) mbar_wait(&bar[q & 1], (q >> 1) & 1, status, &never);
+    if (product_out) mbar_wait(&bar[2], q & 1, status, &never);
   }
+  tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
@@ -881,51 +861,40 @@ __global__ void __launch_bounds__(128, 2)
   }
 }
 
-template <int MW, int NL, bool LCOL>
-int launch_crt_fuse_v(const OzakiArgs &a, const CrtFuse &F, const CUtensorMap &map, int per_sm,
+template <int MW, int NL>
+int launch_crt_fuse_t(const OzakiArgs &a, const CrtFuse &F, const CUtensorMap &map,
                       cudaStream_t s) {
+  const size_t smem = fuse_smem(F.D, NL);
+  if (2 * NL > ((F.D + 15) & ~15))                 // a buffer holds the limb columns
+    return fail(MW_EUNSUPPORTED, "residue form: %d limbs of %d moduli", NL, F.D);
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(crt_fuse_kernel<MW, NL, LCOL>,
+    cudaError_t e = cudaFuncSetAttribute(crt_fuse_kernel<MW, NL>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)fuse_smem(kCrtMaxModuli, NL, LCOL));
+                                         (int)fuse_smem(kCrtMaxModuli, NL));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(crt_fuse_kernel<MW, NL, LCOL>,
+      e = cudaFuncSetAttribute(crt_fuse_kernel<MW, NL>,
                                cudaFuncAttributePreferredSharedMemoryCarveout,
                                cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return cuda_fail(e, "reconstruction smem attribute");
     attr = true;
   }
-  int dev = 0, nsm = 0;
+  int dev = 0, nsm = 0, smem_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t ntiles = (a.N + 127) / 128 * a.M;
-  const unsigned grid = (unsigned)std::min<int64_t>(ntiles, (int64_t)per_sm * nsm);
-  crt_fuse_kernel<MW, NL, LCOL><<<grid, 128, fuse_smem(F.D, NL, LCOL), s>>>(
-      map, a.eA, a.eB, a.M, a.N, 4 - a.S_A - a.S_B, a.C, a.ldc, a.psc, status_ptr(), F);
-  return cuda_fail(cudaGetLastError(), "residue reconstruction launch");
-}
-
-template <int MW, int NL>
-int launch_crt_fuse_t(const OzakiArgs &a, const CrtFuse &F, const CUtensorMap &map,
-                      cudaStream_t s) {
-  int dev = 0, smem_sm = 0;
-  cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, crt_fuse_kernel<MW, NL, false>);
+  cudaError_t e = cudaFuncGetAttributes(&fa, crt_fuse_kernel<MW, NL>);
   if (e != cudaSuccess) return cuda_fail(e, "reconstruction attributes");
-  // resident CTAs: what shared memory (1 KB reserved per CTA), registers and the
-  // tensor memory (512 columns) hold; the limb columns leave shared memory only
-  // when that lets more CTAs reside
-  const int by_regs = ctas_by_registers(fa.numRegs, 128);
-  const int by_tmem = (int)(512 / FuseShape<NL>::TCOLS);
-  const int cap = std::min(by_regs, by_tmem);
-  const int in_smem = smem_sm / (int)(fuse_smem(F.D, NL, false) + 1024);
-  const int in_local = smem_sm / (int)(fuse_smem(F.D, NL, true) + 1024);
-  if (std::min(in_local, cap) > std::min(in_smem, cap))
-    return launch_crt_fuse_v<MW, NL, true>(a, F, map, std::max(1, std::min(in_local, cap)), s);
-  return launch_crt_fuse_v<MW, NL, false>(a, F, map, std::max(1, std::min(in_smem, cap)), s);
+  // resident CTAs: shared memory (1 KB reserved per CTA), registers, tensor memory
+  const int per_sm = std::max(1, std::min({smem_sm / (int)(smem + 1024),
+                                           ctas_by_registers(fa.numRegs, 128),
+                                           (int)(512 / FuseShape<NL>::TCOLS)}));
+  const int64_t ntiles = (a.N + 127) / 128 * a.M;
+  const unsigned grid = (unsigned)std::min<int64_t>(ntiles, (int64_t)per_sm * nsm);
+  crt_fuse_kernel<MW, NL><<<grid, 128, smem, s>>>(map, a.eA, a.eB, a.M, a.N, 4 - a.S_A - a.S_B,
+                                                  a.C, a.ldc, a.psc, status_ptr(), F);
+  return cuda_fail(cudaGetLastError(), "residue reconstruction launch");
 }
 
 template <int MW>
@@ -1030,28 +999,33 @@ int launch_crt_combine(const OzakiArgs &a, cudaStream_t s) {
     }
     if (carry) return fail(MW_EUNSUPPORTED, "residue form: Q' past its limbs");
   }
-  uint64_t borrow = 0;                               // nP = 2^(32 NL) - P
+  F.byte1 = 1u << 8;
+  F.byte2 = 1u << 16;
+  F.byte3 = 1u << 24;
+  uint64_t carry = 0, bias = 0, borrow = 0;
   for (int l = 0; l < NL; ++l) {
-    const uint32_t pl = (size_t)l < P.size() ? P[l] : 0u;
-    F.P[l] = pl;
-    const uint64_t d = (uint64_t)0 - pl - borrow;
-    F.nP[l] = (uint32_t)d;
-    borrow = (pl | borrow) ? 1 : 0;
+    const uint64_t x = (l < (int)P.size() ? P[l] : 0u) + carry;   // balanced limbs of P
+    carry = x >= 0x80000000ull;
+    F.P[l] = (int32_t)(uint32_t)x;
+    bias += 0x4B400000ull * 0x01010101ull;           // minus the bias of every byte position
+    const uint64_t d = (uint64_t)0 - (uint32_t)bias - borrow;
+    F.bias[l] = (uint32_t)d;
+    borrow = ((uint32_t)bias | borrow) ? 1 : 0;
+    bias >>= 32;
   }
   // P ~ Pd 2^e from its top limbs
   double Pd = 0;
   const int lo = std::max(0, (int)P.size() - 3);
   for (int l = (int)P.size() - 1; l >= lo; --l) Pd = Pd * 4294967296.0 + (double)P[l];
   const int e = 32 * lo;
-  F.c64 = (float)std::ldexp(1.0 / Pd, 32 * (top - 1) - e);
-  F.c32 = (float)std::ldexp(1.0 / Pd, 32 * (top - 2) - e);
+  for (int i = 0; i < 8; ++i) F.cz[i] = (float)std::ldexp(1.0 / Pd, 8 * (4 * top - 8 + i) - e);
   // residues: bf16 planes [t][i][j], rows of crt_ld(N); boxes of 64 outputs of
   // one row x every modulus (moduli past D, outputs past N: zeros)
   alignas(64) CUtensorMap map;
   const int64_t ld = crt_ld(a.N);
   const uint64_t dims[3] = {(uint64_t)a.N, (uint64_t)a.M, (uint64_t)D};
   const uint64_t strides[2] = {(uint64_t)ld * 2, (uint64_t)a.M * ld * 2};
-  const uint32_t box[3] = {64, 1, (uint32_t)((D + 7) & ~7)};
+  const uint32_t box[3] = {64, 1, (uint32_t)((D + 15) & ~15)};
   int rc = make_map_bf16(&map, a.partials, 3, dims, strides, box);
   if (rc) return rc;
   switch (a.m) {

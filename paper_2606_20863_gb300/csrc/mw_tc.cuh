@@ -114,23 +114,12 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t *v) {
       : "r"(taddr));
 }
 
-// Four 8 x 8 matrices of 16-bit elements, transposed on the way (ldmatrix .trans):
-// lanes 8j..8j+7 give the addresses of the 16-byte rows of matrix j; thread l
-// receives in register j the elements (row 2(l%4), column l/4) and (row
-// 2(l%4)+1, column l/4) of matrix j, low half first.
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr)
-               : "memory");
-}
-// Four 8 x 8 matrices of 16-bit elements (stmatrix): lanes 8j..8j+7 give the
-// addresses of the rows of matrix j; register j of thread l holds (row l/4,
-// columns 2(l%4), 2(l%4)+1) of matrix j.
-__device__ __forceinline__ void stsm_x4(uint32_t addr, const uint32_t (&r)[4]) {
-  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
-               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
-               : "memory");
+// 32 lanes x 8 columns of 32-bit words.
+__device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t *v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+                 "=r"(v[6]), "=r"(v[7])
+               : "r"(taddr));
 }
 
 // Tensor-memory columns for the CTA (one warp, all lanes): the base address is
@@ -167,6 +156,15 @@ __host__ __device__ __forceinline__ uint32_t sw128_offset(uint32_t row, uint32_t
 __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+// An operand with M (or N) contiguous, 128-byte swizzle: 64 elements of one k in a
+// 128-byte row, eight k 1024 bytes (the stride byte offset), the next 64 elements
+// `group` bytes on (the leading byte offset); what a 128-byte-swizzled TMA box of
+// 64 x k leaves behind.
+__device__ __forceinline__ uint64_t mn128_desc(uint32_t saddr, uint32_t group) {
+  return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(group >> 4) << 16) |
+         ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
 // Instruction descriptor of kind::f16 for an M x N tile: fp32 accumulator
