@@ -9,7 +9,8 @@
 //      again in the rare case of input that is not normalised);
 //   2. every entry cut into S balanced digits of w = 24 bits (|d| <= 2^23) on
 //      the fixed-point grid below 2^E, as for the matrix product (m >= 8:
-//      through a shared-memory column of 24-bit slots, cut_column);
+//      through a shared-memory column of 24-bit slots, cut_column; m <= 4: in as
+//      few 32-bit limbs as the digits need, dot_cut);
 //   3. each thread sums d^a_p d^b_q into int64 diagonal sums s_t, t = p + q < D
 //      (|d^a d^b| <= 2^46, so a thread's share of K stays far below 2^63); the
 //      block adds them up in 128 bits;
@@ -17,6 +18,12 @@
 //      X 2^(E_a + E_b + 4 - w (D+1)) into m words (greedy, ties to even).
 // S is a template parameter (digit positions known at compile time); the
 // planner picks the smallest instance that covers the error analysis.
+//
+// Bound by integer issue, the cut above all: 1,024 products of length 6,144, us,
+// before (64-bit limbs rounded up to pairs, range checked digit by digit, products
+// past the kept diagonals issued and masked) and now: m = 2 212 / 167, m = 4
+// 400 / 292, m = 8 603 / 500, m = 16 1,845 / 1,475 (L2 flushed).  128 threads a CTA:
+// m = 2 195, m = 8 486; 5,000 products of length 500 148 -> 117, not taken.
 //
 // The same kernel multiplies truncated power series (mw_convolve_batched):
 // coefficient i of the product of series s, c_i = sum_{k<=i} a_k b_{i-k}, is the
@@ -73,7 +80,7 @@ __device__ __forceinline__ void add_shifted_u(uint64_t (&X)[NL], uint64_t V, int
   }
 }
 
-template <int MW, int S, int NL, int NLF>
+template <int MW, int S, int NLF>
 __global__ void __launch_bounds__(kDotThreads) dot_kernel(const DotArgs a) {
   constexpr int DC = S + kDotExtraD;
   __shared__ int red_i[4][kDotThreads / 32];
@@ -84,8 +91,8 @@ __global__ void __launch_bounds__(kDotThreads) dot_kernel(const DotArgs a) {
   // [2]: an entry outside the range of its digits (raised after the last cut)
   __shared__ int red_flag[3];
   __shared__ uint32_t rcol[2 * NLF];   // the fusing thread's limbs
-  extern __shared__ double stage[];   // [2 buffers][2 MW words][kDotThreads], then for
-                                      // m >= 8 the threads' digit columns
+  extern __shared__ double stage[];   // m >= 8: [2 buffers][2 MW words][kDotThreads], then
+                                      // the threads' digit columns
   // m >= 8: each word adds its fields into this thread's column of slots
   // (cut_column) instead of a carry chain over every limb
   constexpr bool kColumn = MW >= 8;
@@ -132,8 +139,9 @@ __global__ void __launch_bounds__(kDotThreads) dot_kernel(const DotArgs a) {
     // largest word, as defined); where a later word exceeds the leading words'
     // exponent (input that is not normalised) the vectors are cut again with it.
     int64_t s[DC];
-    // the words of the next entry are copied into this thread's shared slots
-    // while the current one is cut (each thread reads only what it copied)
+    // the words of the next entry load while the current one is cut: m >= 8 copies
+    // them into this thread's shared slots (each thread reads only what it copied),
+    // shorter entries wait in registers
     auto slot = [&](int buf, int j) { return stage + ((buf * 2 * MW + j) * kDotThreads + tid); };
     auto fetch = [&](int64_t k, int buf) {
 #pragma unroll
@@ -142,66 +150,76 @@ __global__ void __launch_bounds__(kDotThreads) dot_kernel(const DotArgs a) {
         cp_async8(slot(buf, MW + j), pb + j * a.psb + k * bs);
       }
     };
+    double na_[kColumn ? 1 : MW], nb_[kColumn ? 1 : MW];
+    auto load = [&](int64_t k) {
+      if constexpr (!kColumn) {
+#pragma unroll
+        for (int j = 0; j < MW; ++j) {
+          na_[j] = pa[j * a.psa + k];
+          nb_[j] = pb[j * a.psb + k * bs];
+        }
+      }
+    };
     for (int attempt = 0; attempt < 2; ++attempt) {
       const int Ea = exps[0], Eb = exps[1];
       const int Fa = kDotW * S - 2 - Ea, Fb = kDotW * S - 2 - Eb;
       int xa_max = kExpZero, xb_max = kExpZero, na = -kExpZero, nb = -kExpZero;
-      bool nonfinite = false;
+      bool nonfinite = false, in_range = true;
 #pragma unroll
       for (int t = 0; t < DC; ++t) s[t] = 0;
       int buf = 0;
-      if (tid < Ki) fetch(tid, 0);
-      cp_async_commit();
-      for (int64_t k = tid; k < Ki; k += kDotThreads, buf ^= 1) {
-        if (k + kDotThreads < Ki) fetch(k + kDotThreads, buf ^ 1);
+      if constexpr (kColumn) {
+        if (tid < Ki) fetch(tid, 0);
         cp_async_commit();
-        cp_async_wait<1>();
+      } else {
+        if (tid < Ki) load(tid);
+      }
+      for (int64_t k = tid; k < Ki; k += kDotThreads, buf ^= 1) {
         double xa[MW], xb[MW];
-        // each entry's largest word: the largest bit pattern without the sign
-        // (the order of non-negative doubles), one exponent per entry
-        uint64_t ma = 0, mb = 0;
+        if constexpr (kColumn) {
+          if (k + kDotThreads < Ki) fetch(k + kDotThreads, buf ^ 1);
+          cp_async_commit();
+          cp_async_wait<1>();
 #pragma unroll
-        for (int j = 0; j < MW; ++j) {
-          xa[j] = *slot(buf, j);
-          xb[j] = *slot(buf, MW + j);
-          const uint64_t ua = (uint64_t)__double_as_longlong(xa[j]) & 0x7FFFFFFFFFFFFFFFull;
-          const uint64_t ub = (uint64_t)__double_as_longlong(xb[j]) & 0x7FFFFFFFFFFFFFFFull;
-          ma = ua > ma ? ua : ma;
-          mb = ub > mb ? ub : mb;
+          for (int j = 0; j < MW; ++j) {
+            xa[j] = *slot(buf, j);
+            xb[j] = *slot(buf, MW + j);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < MW; ++j) {
+            xa[j] = na_[j];
+            xb[j] = nb_[j];
+          }
+          if (k + kDotThreads < Ki) load(k + kDotThreads);
         }
-        const int xa_e = exp_plus1(__longlong_as_double((long long)ma));
-        const int xb_e = exp_plus1(__longlong_as_double((long long)mb));
+        const int xa_e = entry_exp<MW>(xa), xb_e = entry_exp<MW>(xb);
         if (xa_e == kExpNonFinite || xb_e == kExpNonFinite) nonfinite = true;
         if (xa_e != kExpZero && xa_e != kExpNonFinite) { xa_max = max(xa_max, xa_e); na = min(na, xa_e); }
         if (xb_e != kExpZero && xb_e != kExpNonFinite) { xb_max = max(xb_max, xb_e); nb = min(nb, xb_e); }
         int32_t da[S], db[S];
         if constexpr (kColumn) {
-          bool ok = cut_column<MW, kDotW>(xa, Fa, S, dcol, kDotThreads,
-                                          [&](int k, int32_t d) { da[S - 1 - k] = d; });
-          ok &= cut_column<MW, kDotW>(xb, Fb, S, dcol, kDotThreads,
-                                      [&](int k, int32_t d) { db[S - 1 - k] = d; });
-          if (!ok) red_flag[2] = 1;
+          in_range &= cut_column<MW, kDotW>(xa, Fa, S, dcol, kDotThreads,
+                                            [&](int k, int32_t d) { da[S - 1 - k] = d; });
+          in_range &= cut_column<MW, kDotW>(xb, Fb, S, dcol, kDotThreads,
+                                            [&](int k, int32_t d) { db[S - 1 - k] = d; });
         } else {
-          bool ok = true;
-          {
-            uint64_t T[NL];
-            fixed_point<MW, NL>(xa, Fa, T);
-            ok &= dot_digits<S, NL>(T, da);
-          }
-          {
-            uint64_t T[NL];
-            fixed_point<MW, NL>(xb, Fb, T);
-            ok &= dot_digits<S, NL>(T, db);
-          }
-          if (!ok) red_flag[2] = 1;
+          in_range &= dot_cut<MW, S>(xa, Fa, da);
+          in_range &= dot_cut<MW, S>(xb, Fb, db);
         }
 #pragma unroll
         for (int p = 0; p < S; ++p)
 #pragma unroll
-          for (int q = 0; q < S; ++q)
-            if (p + q < DC && p + q < D) s[p + q] += (int64_t)da[p] * (int64_t)db[q];
+          for (int q = 0; q < S - p; ++q) s[p + q] += (int64_t)da[p] * (int64_t)db[q];
+#pragma unroll
+        for (int t = S; t < DC; ++t)
+          if (t < D) {
+#pragma unroll
+            for (int p = t - S + 1; p < S; ++p) s[t] += (int64_t)da[p] * (int64_t)db[t - p];
+          }
       }
-      cp_async_wait<0>();
+      if (!in_range) red_flag[2] = 1;
+      if constexpr (kColumn) cp_async_wait<0>();
       // exponents over all words: the same as the leading words' for normalised
       // input; otherwise cut again (at most once: the second pass uses them)
       for (int o = 16; o; o >>= 1) {
@@ -282,23 +300,23 @@ __global__ void __launch_bounds__(kDotThreads) dot_kernel(const DotArgs a) {
 
 template <int MW, int S>
 int launch_dot_s(const DotArgs &a, cudaStream_t st) {
-  constexpr int NL = 2 * ((kDotW * S + 3 + 127) / 128);   // carry chains exist for even NL
   // |X| < 2^(128 + w (D-1)), D <= S + kDotExtraD
   constexpr int NLF = (128 + kDotW * (S + kDotExtraD - 1) + 1 + 63) / 64;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int grid = (int)std::min<int64_t>(a.conv ? a.count * a.K : a.count, (int64_t)nsm * 8);
-  constexpr size_t smem = 2 * 2 * MW * kDotThreads * sizeof(double) +
-                         (MW >= 8 ? (size_t)(S + 3) * kDotThreads * sizeof(uint32_t) : 0);
+  constexpr size_t smem = MW >= 8 ? 2 * 2 * MW * kDotThreads * sizeof(double) +
+                                        (size_t)(S + 3) * kDotThreads * sizeof(uint32_t)
+                                  : 0;
   static bool attr_set = false;   // once per instance
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(dot_kernel<MW, S, NL, NLF>,
+    cudaError_t e = cudaFuncSetAttribute(dot_kernel<MW, S, NLF>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "dot kernel smem attribute");
     attr_set = true;
   }
-  dot_kernel<MW, S, NL, NLF><<<grid, kDotThreads, smem, st>>>(a);
+  dot_kernel<MW, S, NLF><<<grid, kDotThreads, smem, st>>>(a);
   return cuda_fail(cudaGetLastError(), "dot kernel launch");
 }
 

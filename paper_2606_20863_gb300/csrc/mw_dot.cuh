@@ -6,7 +6,7 @@
 
 #include "mw_device.cuh"
 #include "mw_internal.h"
-#include "mw_pieces.cuh"
+#include "mw_limbs.cuh"
 
 namespace mw {
 
@@ -41,47 +41,86 @@ int launch_series(int m, int S, const DotArgs &a, cudaStream_t st);
 
 namespace {
 
-// bits 24k + 23 for k = 0 .. S-2 (the bias that makes the low digits bytes-like)
+// 32-bit limbs of a fixed-point value of S digits (|T| < 2^(24 S + 1), a sign bit).
+__host__ __device__ constexpr int dot_limbs(int S) { return (kDotW * S + 3 + 31) / 32 < 4 ? 4 : (kDotW * S + 3 + 31) / 32; }
+
+// limb i of H = sum of 2^(24k + 23) for k = 0 .. S-2: adding it makes the low digits
+// plain 24-bit fields
 template <int S>
-__host__ __device__ constexpr uint64_t dot_bias(int limb) {
-  uint64_t v = 0;
+__host__ __device__ constexpr uint32_t dot_bias(int limb) {
+  uint32_t v = 0;
   for (int k = 0; k + 1 < S; ++k) {
     const int bit = kDotW * k + kDotW - 1;
-    if (bit / 64 == limb) v |= 1ull << (bit % 64);
+    if (bit / 32 == limb) v |= 1u << (bit % 32);
   }
   return v;
 }
 
-// Balanced digits d[p] (p = 0 most significant) of the NL-limb fixed-point
-// value T, w = 24: with 2^23 added to every low digit the digits are 24-bit
-// fields minus 2^23; the top digit is the signed value above them.  Returns
-// false when T lies outside [-2^(wS-1), 2^(wS-1)).
-template <int S, int NL>
-__device__ __forceinline__ bool dot_digits(uint64_t (&T)[NL], int32_t (&d)[S]) {
-  constexpr int b = kDotW * S - 1, lb = b >> 6, ob = b & 63;
-  static_assert(lb < NL, "limbs cover the digits");
-  const int64_t v = (int64_t)T[lb] >> ob;
-  bool ok = v == 0 || v == -1;
+// Balanced digits d[p] (p = 0 most significant) of T = sum_j trunc(x_j 2^F), w = 24:
+// 24-bit fields of T + H minus 2^23; the top digit is the signed value above
+// them.  Returns false when T lies outside [-2^(wS-1), 2^(wS-1)): certainly inside
+// when the first word's exponent is covered (F = wS - 2 - E) and the later words
+// lie log2(MW) binary orders below it, else checked on the digits.
+template <int MW, int S>
+__device__ __forceinline__ bool dot_cut(const double (&x)[MW], int F, int32_t (&d)[S]) {
+  constexpr int NL = dot_limbs(S);
+  uint32_t T[NL];
 #pragma unroll
-  for (int i = lb + 1; i < NL; ++i) ok &= T[i] == (uint64_t)v;
-  uint64_t H[NL];
+  for (int i = 0; i < NL; ++i) T[i] = dot_bias<S>(i);
+  const uint32_t h0 = (uint32_t)__double2hiint(x[0]) << 1;
+  uint32_t h1 = 0;
 #pragma unroll
-  for (int i = 0; i < NL; ++i) H[i] = dot_bias<S>(i);
-  add_limbs<NL>(T, H);
+  for (int j = 0; j < MW; ++j) {
+    if (j) h1 = max(h1, (uint32_t)__double2hiint(x[j]) << 1);
+    add_word32<NL>(x[j], F, T);
+  }
+  int lsign = 0;
+  constexpr uint32_t kGap = MW <= 2 ? 1 : 2;
+  static_assert(MW <= 4, "gap of the later words");
+  const bool plain = (h1 >> 21) + kGap <= (h0 >> 21) && (int)(h0 >> 21) - 1022 <= kDotW * S - 2 - F;
 #pragma unroll
   for (int k = 0; k < S; ++k) {          // k: position from the least significant digit
-    const int bit = kDotW * k, li = bit >> 6, off = bit & 63;
-    uint64_t win = T[li] >> off;
-    if (off != 0 && li + 1 < NL) win |= T[li + 1] << (64 - off);
+    const int bit = kDotW * k, li = bit >> 5, off = bit & 31;
+    uint32_t win = T[li] >> off;
     if (k + 1 < S) {
-      d[S - 1 - k] = (int32_t)(win & 0xFFFFFF) - (1 << 23);
-    } else {
-      // the top digit: everything from bit 24 (S-1) up, sign included
-      const int64_t top = (li + 1 < NL || off == 0) ? (int64_t)win : ((int64_t)T[li] >> off);
-      d[0] = (int32_t)top;
+      if (off > 8) win |= T[li + 1] << (32 - off);
+      d[S - 1 - k] = (int32_t)(win & 0xFFFFFFu) - (1 << 23);
+    } else {                             // everything from bit 24 (S-1) up, sign included
+      d[0] = li + 1 < NL ? (int32_t)__funnelshift_r(T[li], T[li + 1], off)
+                         : (int32_t)T[li] >> off;
     }
   }
-  return ok;
+  if (plain) return true;
+  // T = top 2^(w(S-1)) + L with L of the sign of its highest nonzero digit: in range for
+  // |top| < 2^(w-1), for top = -2^(w-1) with L >= 0 and top = 2^(w-1) with L < 0
+#pragma unroll
+  for (int k = 0; k + 1 < S; ++k)
+    if (d[S - 1 - k] != 0) lsign = d[S - 1 - k] > 0 ? 1 : -1;
+  constexpr int top_bits = 32 * NL - kDotW * (S - 1);            // bits of the top field
+  bool above = true;                                             // they extend d[0]'s sign
+  if constexpr (top_bits > 32) {
+    constexpr int li = kDotW * (S - 1) / 32, off = kDotW * (S - 1) % 32;
+    static_assert(li + 1 == NL - 1, "the top field ends in the last limb");
+    above = ((int32_t)T[NL - 1] >> off) == (d[0] >> 31);
+  }
+  constexpr int half = 1 << 23;
+  return above && ((d[0] > -half && d[0] < half) || (d[0] == -half && lsign >= 0) ||
+                   (d[0] == half && lsign < 0));
+}
+
+// ilogb + 1 of the largest word of an entry (kExpZero, kExpNonFinite as exp_plus1):
+// the largest high word without its sign holds it unless it is zero, subnormal or not finite.
+template <int MW>
+__device__ __forceinline__ int entry_exp(const double (&x)[MW]) {
+  uint32_t h = 0;
+#pragma unroll
+  for (int j = 0; j < MW; ++j) h = max(h, (uint32_t)__double2hiint(x[j]) << 1);
+  const int be = (int)(h >> 21);
+  if (be != 0 && be != 0x7ff) return be - 1022;
+  int e = kExpZero;
+#pragma unroll
+  for (int j = 0; j < MW; ++j) e = max(e, exp_plus1(x[j]));      // non-finite: the largest
+  return e;
 }
 
 }  // namespace

@@ -19,9 +19,10 @@
 // Row r has 32 (r + 1) steps, so a warp takes rows r and R - 1 - r; with few
 // series `ks` warps share a row's k and add their sums in shared memory.
 //
-// Bound by the 32 x 32 -> 64 bit multiply-adds.  One CTA per coefficient (which
-// cuts i + 1 entries of both series again for each) took 17.25 ms for 2,000
-// octo-double pairs of degree 127.
+// Bound by the 32 x 32 -> 64 bit multiply-adds (133 M warp instructions for 2,000
+// octo-double pairs of degree 127, about four cycles each and SM sub-partition:
+// 0.45 ms): those pairs take 0.63 ms, and took 17.25 ms with one CTA per coefficient
+// (which cuts i + 1 entries of both series again for each).
 #include <cuda.h>
 
 #include <algorithm>
@@ -38,7 +39,6 @@ constexpr size_t kSeriesSmem = 232448;             // shared memory a CTA can ha
 template <int MW, int S> struct SeriesShape {
   static constexpr int DC = S + kDotExtraD;
   static constexpr int SP = (S + 3) / 4 * 4;       // a's digits of one entry, in int4
-  static constexpr int NL = 2 * ((kDotW * S + 3 + 127) / 128);
   static constexpr int NL32 = (kDotW * (DC - 1) + 65 + 31) / 32;   // |X| < 2^(64 + w (D-1))
   // column of a thread: the slots of cut_column (m >= 8), then the rounding's limbs
   static constexpr int COL = (MW >= 8 && S + 3 > NL32) ? S + 3 : NL32;
@@ -58,7 +58,7 @@ template <int MW, int S>
 __global__ void __launch_bounds__(32 * kSeriesWarps, MW == 16 ? 1 : 2)
     series_kernel(const DotArgs a, int ks, int pairs, int parts) {
   using SH = SeriesShape<MW, S>;
-  constexpr int DC = SH::DC, SP = SH::SP, NL = SH::NL, NL32 = SH::NL32;
+  constexpr int DC = SH::DC, SP = SH::SP, NL32 = SH::NL32;
   const int n = (int)a.K, nr = (int)series_round32(n), rows = nr / 32;
   const int row_pairs = (rows + 1) / 2, nthr = blockDim.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -88,13 +88,10 @@ __global__ void __launch_bounds__(32 * kSeriesWarps, MW == 16 ? 1 : 2)
       for (int k = tid; k < nr; k += nthr) {
         int e = kExpZero;
         if (k < n) {
-          uint64_t mx = 0;                         // the entry's largest word
+          double x[MW];
 #pragma unroll
-          for (int j = 0; j < MW; ++j) {
-            const uint64_t u = (uint64_t)__double_as_longlong(px[o][j * ps[o] + k]) & 0x7FFFFFFFFFFFFFFFull;
-            mx = u > mx ? u : mx;
-          }
-          e = exp_plus1(__longlong_as_double((long long)mx));
+          for (int j = 0; j < MW; ++j) x[j] = px[o][j * ps[o] + k];
+          e = entry_exp<MW>(x);
           if (e == kExpNonFinite) {
             atomicOr(&flags[3], MW_ENONFINITE);
             e = kExpZero;
@@ -173,13 +170,11 @@ __global__ void __launch_bounds__(32 * kSeriesWarps, MW == 16 ? 1 : 2)
         int32_t *dst = o ? db + 32 + k : da + k * SP;
         const int step = o ? ldb_ : 1;
         if constexpr (MW >= 8) {
-          ok &= cut_column<MW, kDotW>(x, F, S, col, nthr,
-                                      [&](int q, int32_t d) { dst[(S - 1 - q) * step] = d; });
+          ok &= cut_column<MW, kDotW, false>(x, F, S, col, nthr,
+                                             [&](int q, int32_t d) { dst[(S - 1 - q) * step] = d; });
         } else {
-          uint64_t T[NL];
           int32_t d[S];
-          fixed_point<MW, NL>(x, F, T);
-          ok &= dot_digits<S, NL>(T, d);
+          ok &= dot_cut<MW, S>(x, F, d);
 #pragma unroll
           for (int q = 0; q < S; ++q) dst[q * step] = d[q];
         }
