@@ -402,20 +402,11 @@ cudaStream_t side_stream() {
   return st[dev];
 }
 
+// counter: the product kernel's work counter, cleared on the way when *cleared says so.
 int split_both(const mw_plan &p, int transA, int transB, int64_t M, int64_t N, int64_t K,
                const double *A, int64_t lda, int64_t psa, const double *B, int64_t ldb,
-               int64_t psb, void *ws, const Layout &L, bool exps_only, cudaStream_t s) {
-  // residue splits hold tensor memory on every SM they run on: with more than
-  // 64 moduli two of them would not fit side by side, so they run one after the
-  // other on the caller's stream
-  cudaStream_t s2 = (p.mode == MW_CRT && !exps_only && p.D > 64) ? nullptr : side_stream();
-  cudaEvent_t ev[2] = {nullptr, nullptr};
-  bool fork = s2 != nullptr &&
-              cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming) == cudaSuccess;
-  if (fork) fork = cudaEventRecord(ev[0], s) == cudaSuccess &&
-                   cudaStreamWaitEvent(s2, ev[0], 0) == cudaSuccess;
-  if (!fork) s2 = s;
+               int64_t psb, void *ws, const Layout &L, bool exps_only, unsigned long long *counter,
+               bool *cleared, cudaStream_t s) {
   Operands o = ops_in(ws, M, N);
   uint8_t *w8 = static_cast<uint8_t *>(ws);
   SplitArgs a{};
@@ -427,15 +418,41 @@ int split_both(const mw_plan &p, int transA, int transB, int64_t M, int64_t N, i
   a.digits = w8 + L.digA; a.exps = o.eA; a.spread = o.spA; a.max_spread = o.maxsp;
   a.range = p.range_A;
   a.redo = p.mode == MW_CRT ? o.redo : nullptr;
-  int rc = launch_split(a, exps_only, s);
-  if (!rc) {
-    // op(B) used as its transpose: rows N; B stored K x N (trans 0 -> columns) or N x K
-    a.trans = !transB; a.R = N; a.ld = ldb; a.plane_stride = psb; a.X = B; a.S = p.S_B;
-    a.digits = w8 + L.digB; a.exps = o.eB; a.spread = o.spB; a.max_spread = o.maxsp + 1;
-    a.range = p.range_B;
-    a.redo = p.mode == MW_CRT ? o.redo + 1 : nullptr;
-    rc = launch_split(a, exps_only, s2);
+  // op(B) used as its transpose: rows N; B stored K x N (trans 0 -> columns) or N x K
+  SplitArgs b = a;
+  b.trans = !transB; b.R = N; b.ld = ldb; b.plane_stride = psb; b.X = B; b.S = p.S_B;
+  b.digits = w8 + L.digB; b.exps = o.eB; b.spread = o.spB; b.max_spread = o.maxsp + 1;
+  b.range = p.range_B;
+  b.redo = p.mode == MW_CRT ? o.redo + 1 : nullptr;
+  const bool together = exps_together(a, b, exps_only);
+  *cleared = false;
+  if (together) {
+    int rc = launch_exps_pair(a, b, counter, s);
+    if (rc) return rc;
+    *cleared = counter != nullptr;
+    if (exps_only) return MW_OK;
+    if (digits_together(a, b)) return launch_digits(a, &b, s);
   }
+  // the rest of one operand on the given stream
+  auto rest = [&](SplitArgs &x, cudaStream_t st) {
+    if (!together) return launch_split(x, exps_only, st);
+    x.redo = nullptr;
+    x.gate = nullptr;
+    return x.nmod > 0 ? launch_residues(x, st) : launch_digits(x, nullptr, st);
+  };
+  // residue splits hold tensor memory on every SM they run on: with more than
+  // 64 moduli two of them would not fit side by side, so they run one after the
+  // other on the caller's stream
+  cudaStream_t s2 = (p.mode == MW_CRT && !exps_only && p.D > 64) ? nullptr : side_stream();
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  bool fork = s2 != nullptr &&
+              cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming) == cudaSuccess;
+  if (fork) fork = cudaEventRecord(ev[0], s) == cudaSuccess &&
+                   cudaStreamWaitEvent(s2, ev[0], 0) == cudaSuccess;
+  if (!fork) s2 = s;
+  int rc = rest(a, s);
+  if (!rc) rc = rest(b, s2);
   // join the side stream whatever happened (inside a capture a fork must be joined)
   if (fork) {
     cudaError_t e = cudaEventRecord(ev[1], s2);
@@ -480,11 +497,19 @@ int mw_gemm(const mw_plan *plan, int transA, int transB, int64_t M, int64_t N, i
   phase(0, s);
   cudaError_t e = cudaMemsetAsync(ops_in(ws, M, N).maxsp, 0, 2 * sizeof(int32_t), s);
   if (e != cudaSuccess) return cuda_fail(e, "mw_gemm memset");
-  if ((rc = split_both(p, transA, transB, M, N, K, A, lda, psa, B, ldb, psb, ws, L, false, s)))
-    return rc;
-  phase(1, s);
   Operands o = ops_in(ws, M, N);
   uint8_t *w8 = static_cast<uint8_t *>(ws);
+  OzakiArgs oz{};
+  oz.m = p.m; oz.w = p.w; oz.S_A = p.S_A; oz.S_B = p.S_B; oz.D = p.D; oz.group = p.group;
+  oz.chunk = p.chunk; oz.M = M; oz.N = N; oz.Kp = L.Kp;
+  oz.crt = p.mode == MW_CRT;
+  oz.dA = w8 + L.digA; oz.dB = w8 + L.digB; oz.eA = o.eA; oz.eB = o.eB;
+  oz.partials = w8 + L.partials;
+  oz.C = C; oz.ldc = ldc; oz.psc = psc;
+  if ((rc = split_both(p, transA, transB, M, N, K, A, lda, psa, B, ldb, psb, ws, L, false,
+                       p.mode == MW_PLAIN ? nullptr : ozaki_counter(oz), &oz.counter_clear, s)))
+    return rc;
+  phase(1, s);
   if (p.mode == MW_PLAIN) {
     PlainArgs a{};
     a.m = p.m; a.w = p.w; a.S_A = p.S_A; a.S_B = p.S_B; a.D = p.D;
@@ -497,14 +522,7 @@ int mw_gemm(const mw_plan *plan, int transA, int transB, int64_t M, int64_t N, i
     phase(3, s);
     return rc;
   }
-  OzakiArgs a{};
-  a.m = p.m; a.w = p.w; a.S_A = p.S_A; a.S_B = p.S_B; a.D = p.D; a.group = p.group;
-  a.chunk = p.chunk; a.M = M; a.N = N; a.Kp = L.Kp;
-  a.crt = p.mode == MW_CRT;
-  a.dA = w8 + L.digA; a.dB = w8 + L.digB; a.eA = o.eA; a.eB = o.eB;
-  a.partials = w8 + L.partials;
-  a.C = C; a.ldc = ldc; a.psc = psc;
-  rc = launch_ozaki(a, s, [&] { phase(2, s); });
+  rc = launch_ozaki(oz, s, [&] { phase(2, s); });
   phase(3, s);
   return rc;
 }
@@ -544,7 +562,9 @@ int mw_measure_spread(int m, int transA, int transB, int64_t M, int64_t N, int64
   Operands o = ops_in(ws, M, N);
   cudaError_t e = cudaMemsetAsync(o.maxsp, 0, 2 * sizeof(int32_t), s);
   if (e != cudaSuccess) return cuda_fail(e, "measure memset");
-  if ((rc = split_both(p, transA, transB, M, N, K, A, lda, psa, B, ldb, psb, ws, L, true, s)))
+  bool cleared = false;
+  if ((rc = split_both(p, transA, transB, M, N, K, A, lda, psa, B, ldb, psb, ws, L, true, nullptr,
+                       &cleared, s)))
     return rc;
   int32_t host[2];
   if ((e = cudaMemcpyAsync(host, o.maxsp, sizeof host, cudaMemcpyDeviceToHost, s)) != cudaSuccess)

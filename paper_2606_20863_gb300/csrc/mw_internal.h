@@ -35,6 +35,15 @@ struct SplitArgs {
   const int32_t *gate;
 };
 int launch_split(const SplitArgs &a, bool exponents_only, cudaStream_t s);
+// Both operands of a product: whether their exponents are taken in one launch
+// (launch_exps_pair; *max_spread zero before it; clears *counter unless NULL), and
+// whether their digits are cut in one.
+bool exps_together(const SplitArgs &a, const SplitArgs &b, bool exponents_only);
+bool digits_together(const SplitArgs &a, const SplitArgs &b);
+int launch_exps_pair(const SplitArgs &a, const SplitArgs &b, unsigned long long *counter,
+                     cudaStream_t s);
+// Pieces of a (and of *b unless NULL, in the same launch) from their exponents.
+int launch_digits(const SplitArgs &a, const SplitArgs *b, cudaStream_t s);
 
 // ---- plain FP64 form (mw_plain.cu) -------------------------------------------
 struct PlainArgs {
@@ -51,6 +60,7 @@ int launch_plain(const PlainArgs &a, cudaStream_t s);
 struct OzakiArgs {
   int m, w, S_A, S_B, D, group, chunk;
   bool crt;                     // residue form: S_A, S_B fixed-point bits, D moduli
+  bool counter_clear;           // the work counter is zero already
   int64_t M, N, Kp;
   const void *dA, *dB;          // bf16 pieces, S x rows x Kp
   const int32_t *eA, *eB;
@@ -77,7 +87,8 @@ struct ProductLaunch {
   void *partials;                 // int32 [t][M][N] (narrow) or int64 [g][M][N]
   bool narrow;
   bool crt;                       // residue form: one product per modulus t < D
-  unsigned long long *next_item;  // work counter (reset by launch_product)
+  unsigned long long *next_item;  // work counter
+  bool counter_clear;             // it is zero already (otherwise launch_product clears it)
 };
 int launch_product(const ProductLaunch &a, cudaStream_t s);
 
@@ -85,6 +96,8 @@ int launch_product(const ProductLaunch &a, cudaStream_t s);
 int launch_combine(const OzakiArgs &a, int G, bool narrow, cudaStream_t s);
 // between_kernels runs after the product kernel is launched, before the combine.
 int launch_ozaki(const OzakiArgs &a, cudaStream_t s, const std::function<void()> &between_kernels);
+// Where launch_ozaki keeps the product kernel's work counter (behind the partial sums).
+unsigned long long *ozaki_counter(const OzakiArgs &a);
 // Every diagonal sum s_t fits in int32: S_min * K * 2^(2w-2) < 2^31.  Then the
 // partial sums are the int32 s_t, otherwise int64 group sums; every plane is
 // column-major (entry (i, j) at j M + i).

@@ -813,8 +813,10 @@ int launch_product(const ProductLaunch &a, cudaStream_t s) {
     if (e != cudaSuccess) return cuda_fail(e, "product kernel smem attribute");
     attr_set = true;
   }
-  cudaError_t e = cudaMemsetAsync(a.next_item, 0, sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return cuda_fail(e, "work counter reset");
+  if (!a.counter_clear) {
+    cudaError_t e = cudaMemsetAsync(a.next_item, 0, sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return cuda_fail(e, "work counter reset");
+  }
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -862,6 +864,14 @@ size_t ozaki_partials_bytes(int64_t M, int64_t N, int D, int group, bool narrow)
   return ((planes + 255) & ~(size_t)255) + 256;
 }
 
+unsigned long long *ozaki_counter(const OzakiArgs &a) {
+  const bool narrow = a.crt || narrow_partials(a.S_A, a.S_B, a.w, a.Kp);
+  const size_t planes = a.crt ? crt_residue_planes_bytes(a.M, a.N, a.D)
+                              : ozaki_partials_planes_bytes(a.M, a.N, a.D, a.group, narrow);
+  return reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(a.partials) +
+                                                ((planes + 255) & ~(size_t)255));
+}
+
 int launch_ozaki(const OzakiArgs &a, cudaStream_t s, const std::function<void()> &between_kernels) {
   if (a.Kp % BK) return fail(MW_EINVAL, "padded K must be a multiple of %d", BK);
   const int G = n_groups(a.D, a.group);
@@ -881,10 +891,8 @@ int launch_ozaki(const OzakiArgs &a, cudaStream_t s, const std::function<void()>
   L.M = a.M; L.N = a.N; L.K = a.Kp;
   L.partials = a.partials;
   L.narrow = narrow;
-  const size_t planes = a.crt ? crt_residue_planes_bytes(a.M, a.N, a.D)
-                              : ozaki_partials_planes_bytes(a.M, a.N, a.D, a.group, narrow);
-  L.next_item = reinterpret_cast<unsigned long long *>(
-      reinterpret_cast<uint8_t *>(a.partials) + ((planes + 255) & ~(size_t)255));
+  L.next_item = ozaki_counter(a);
+  L.counter_clear = a.counter_clear;
   int rc = launch_product(L, s);
   if (rc) return rc;
   if (between_kernels) between_kernels();

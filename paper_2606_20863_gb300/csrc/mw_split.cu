@@ -141,14 +141,112 @@ __global__ void exps_finalize_kernel(int64_t R, int *E, int *spread, int *max_sp
   if (range >= 0 && sp > range) raise_status(status, MW_WRANGE);
 }
 
+// Pass 1 of both operands of a product in one launch: no atomics on the rows, no
+// clearing, no finalize, no second stream.  trans = 0: a warp per row, eight rows a
+// block; trans = 1: 8 columns x 32 rows of the stored matrix at a time; either way
+// the threads that see a row or column see all of it, so reductions are short
+// (kPairMaxK) and, in a product, operands small (kPairMaxWords: 384^3 quad doubles 120
+// -> 114 us, 512^3 149 -> 159, 256^3 octo doubles 150 -> 137, 384^3 236 -> 246; above
+// that the two-stream passes over chunks keep more loads in flight).  The spread
+// measurement, which waits for the result, always takes it (2048 x 1024 double
+// doubles: 96 -> 46 us a call).  The first block clears the product kernel's work
+// counter.
+constexpr int64_t kPairMaxK = 2048;
+constexpr int64_t kPairMaxWords = 3 << 19;
+constexpr int kPairCols = 8;
+struct ExpsArgs {
+  const double *X;
+  int64_t R, K, ld, ps;
+  int trans, range;
+  int32_t *E, *spread, *max_spread;
+};
+__host__ __device__ __forceinline__ int64_t exps_pair_blocks(const ExpsArgs &a) { return (a.R + 7) / 8; }
+
+template <int MW>
+__device__ __forceinline__ void exps_entry(const double *x, int64_t ps, int &emax, int &emin,
+                                           bool &bad) {
+  double v[MW];
+  uint32_t h = 0;                                  // largest high word without its sign
+#pragma unroll
+  for (int j = 0; j < MW; ++j) v[j] = x[j * ps];
+#pragma unroll
+  for (int j = 0; j < MW; ++j) h = max(h, (uint32_t)__double2hiint(v[j]) << 1);
+  int e = (int)(h >> 21) - 1022;
+  if ((h >> 21) == 0 || (h >> 21) == 0x7ff) {      // zero, subnormal or not finite
+    e = kExpZero;
+#pragma unroll
+    for (int j = 0; j < MW; ++j) {
+      const int u = exp_plus1(v[j]);
+      if (u == kExpNonFinite) bad = true;
+      else e = max(e, u);
+    }
+  }
+  if (e != kExpZero) {
+    emax = max(emax, e);
+    emin = min(emin, e);
+  }
+}
+
+template <int MW>
+__global__ void __launch_bounds__(256) exps_pair_kernel(ExpsArgs a, ExpsArgs b, unsigned blocks_a,
+                                                        unsigned long long *counter,
+                                                        unsigned int *status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && counter) *counter = 0;
+  const bool second = blockIdx.x >= blocks_a;
+  const ExpsArgs &p = second ? b : a;
+  const int64_t r0 = 8 * (int64_t)(blockIdx.x - (second ? blocks_a : 0u));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int emax = kExpZero, emin = -kExpZero;
+  bool bad = false;
+  auto finish = [&](int64_t r) {                   // one thread per row
+    const int Er = emax == kExpZero ? 0 : emax, sp = emax == kExpZero ? 0 : emax - emin;
+    p.E[r] = Er;
+    p.spread[r] = sp;
+    if (sp > 0) atomicMax(p.max_spread, sp);
+    if (p.range >= 0 && sp > p.range) raise_status(status, MW_WRANGE);
+  };
+  if (!p.trans) {
+    const int64_t r = r0 + warp;
+    if (r < p.R)
+#pragma unroll(MW <= 4 ? 4 : 1)
+      for (int64_t k = lane; k < p.K; k += 32)
+        exps_entry<MW>(p.X + r * p.ld + k, p.ps, emax, emin, bad);
+    for (int o = 16; o; o >>= 1) {
+      emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+      emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
+    }
+    if (lane == 0 && r < p.R) finish(r);
+  } else {
+    __shared__ int smax[32][kPairCols], smin[32][kPairCols];
+    const int tx = threadIdx.x % kPairCols, ty = threadIdx.x / kPairCols;
+    const int64_t r = r0 + tx;
+    if (r < p.R)
+#pragma unroll(MW <= 4 ? 4 : 1)
+      for (int64_t k = ty; k < p.K; k += 32)
+        exps_entry<MW>(p.X + k * p.ld + r, p.ps, emax, emin, bad);
+    smax[ty][tx] = emax;
+    smin[ty][tx] = emin;
+    __syncthreads();
+    if (threadIdx.x < kPairCols && r < p.R) {
+      for (int i = 1; i < 32; ++i) {
+        emax = max(emax, smax[i][tx]);
+        emin = min(emin, smin[i][tx]);
+      }
+      finish(r);
+    }
+  }
+  if (bad) raise_status(status, MW_ENONFINITE);
+}
+
 // ---- pass 2 ------------------------------------------------------------------
 // trans = 0: one thread per (row, pair of columns), pairs cover the padded width.
 template <int MW, int NL, typename Out>
-__global__ void pieces_rows_kernel(const double *__restrict__ X, int64_t R, int64_t K,
-                                   int64_t ld, int64_t ps, int w, int S, Out *digits,
-                                   int64_t dld, const int *E, unsigned int *status) {
+__device__ __forceinline__ void pieces_rows(const double *__restrict__ X, int64_t R, int64_t K,
+                                            int64_t ld, int64_t ps, int w, int S, Out *digits,
+                                            int64_t dld, const int *E, unsigned int *status,
+                                            int64_t block) {
   const int64_t npair = dld / 2;
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t idx = block * 256 + threadIdx.x;
   if (idx >= R * npair) return;
   const int64_t r = idx / npair, k = 2 * (idx % npair);
   double a[MW], b[MW];
@@ -173,15 +271,21 @@ __global__ void pieces_rows_kernel(const double *__restrict__ X, int64_t R, int6
     cut_pair<MW, NL, Out>(a, b, F, w, S, digits + r * dld + k, R * dld, status);
 }
 
+template <int MW, int NL, typename Out>
+__global__ void pieces_rows_kernel(const double *__restrict__ X, int64_t R, int64_t K,
+                                   int64_t ld, int64_t ps, int w, int S, Out *digits,
+                                   int64_t dld, const int *E, unsigned int *status) {
+  pieces_rows<MW, NL, Out>(X, R, K, ld, ps, w, S, digits, dld, E, status, blockIdx.x);
+}
+
 // trans = 1: 32 x 32 tiles (32 rows r, 32 columns k of the logical operand)
 // staged through shared memory as doubles (m planes), then cut like trans = 0.
 template <int MW, int NL, typename Out>
-__global__ void pieces_cols_kernel(const double *__restrict__ X, int64_t R, int64_t K,
-                                   int64_t ld, int64_t ps, int w, int S, Out *digits,
-                                   int64_t dld, const int *E, unsigned int *status) {
-  extern __shared__ double tile[];  // [m][32 k][33]
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  const int64_t r0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
+__device__ __forceinline__ void pieces_cols(const double *__restrict__ X, int64_t R, int64_t K,
+                                            int64_t ld, int64_t ps, int w, int S, Out *digits,
+                                            int64_t dld, const int *E, unsigned int *status,
+                                            int64_t r0, int64_t k0, double *tile) {
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8; tile [m][32 k][33]
 #pragma unroll
   for (int j = 0; j < MW; ++j)
 #pragma unroll
@@ -211,6 +315,68 @@ __global__ void pieces_cols_kernel(const double *__restrict__ X, int64_t R, int6
   }
 }
 
+template <int MW, int NL, typename Out>
+__global__ void __launch_bounds__(256)
+    pieces_cols_kernel(const double *__restrict__ X, int64_t R, int64_t K, int64_t ld, int64_t ps,
+                       int w, int S, Out *digits, int64_t dld, const int *E, unsigned int *status) {
+  extern __shared__ double tile[];
+  pieces_cols<MW, NL, Out>(X, R, K, ld, ps, w, S, digits, dld, E, status, blockIdx.x * (int64_t)32,
+                           blockIdx.y * (int64_t)32, tile);
+}
+
+// Pieces of both operands in one launch, for small products (kPairMaxEntries), where
+// a second stream's fork and join cost more than the kernels beside each other save:
+// with the exponents together 64^3 double doubles 45.6 -> 31.9 us a call (37 -> 25
+// replayed from a graph), 64^3 octo doubles 82.7 -> 66.3.
+constexpr int64_t kPairMaxEntries = 1 << 18;
+template <typename Out> struct PieceArgs {
+  const double *X;
+  int64_t R, K, ld, ps, dld;
+  int trans, S;
+  Out *digits;
+  const int32_t *E;
+};
+template <int MW, int NL, typename Out>
+__global__ void __launch_bounds__(256) pieces_pair_kernel(PieceArgs<Out> a, PieceArgs<Out> b,
+                                                          unsigned blocks_a, int w,
+                                                          unsigned int *status) {
+  extern __shared__ double tile[];
+  const bool second = blockIdx.x >= blocks_a;
+  const PieceArgs<Out> &p = second ? b : a;
+  const int64_t u = blockIdx.x - (second ? blocks_a : 0u);
+  if (!p.trans) {
+    pieces_rows<MW, NL, Out>(p.X, p.R, p.K, p.ld, p.ps, w, p.S, p.digits, p.dld, p.E, status, u);
+  } else {
+    const int64_t nr = (p.R + 31) / 32, kb = u / nr;
+    pieces_cols<MW, NL, Out>(p.X, p.R, p.K, p.ld, p.ps, w, p.S, p.digits, p.dld, p.E, status,
+                             (u - kb * nr) * 32, kb * 32, tile);
+  }
+}
+
+template <int MW, typename Out, int NL>
+int launch_pieces_pair(const SplitArgs &a, const SplitArgs &b, cudaStream_t s) {
+  auto args = [](const SplitArgs &x) {
+    return PieceArgs<Out>{x.X, x.R, x.K, x.ld, x.plane_stride, x.digit_ld, x.trans, x.S,
+                          static_cast<Out *>(x.digits), x.exps};
+  };
+  auto blocks = [](const SplitArgs &x) {
+    return (unsigned)(x.trans ? (x.R + 31) / 32 * ((x.digit_ld + 31) / 32)
+                              : (x.R * (x.digit_ld / 2) + 255) / 256);
+  };
+  const size_t sm = a.trans || b.trans ? (size_t)MW * 32 * 33 * sizeof(double) : 0;
+  static bool attr_set = false;  // once per instantiation
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(pieces_pair_kernel<MW, NL, Out>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         MW * 32 * 33 * (int)sizeof(double));
+    if (e != cudaSuccess) return cuda_fail(e, "split smem attribute");
+    attr_set = true;
+  }
+  pieces_pair_kernel<MW, NL, Out><<<blocks(a) + blocks(b), 256, sm, s>>>(args(a), args(b), blocks(a),
+                                                                        a.w, status_ptr());
+  return cuda_fail(cudaGetLastError(), "split pieces launch");
+}
+
 template <int MW, typename Out, int NL>
 int launch_pieces(const SplitArgs &a, cudaStream_t s) {
   Out *dig = static_cast<Out *>(a.digits);
@@ -229,37 +395,45 @@ int launch_pieces(const SplitArgs &a, cudaStream_t s) {
       if (e != cudaSuccess) return cuda_fail(e, "split smem attribute");
       attr_set = true;
     }
-    pieces_cols_kernel<MW, NL, Out><<<grid, dim3(32, 8), sm, s>>>(
+    pieces_cols_kernel<MW, NL, Out><<<grid, 256, sm, s>>>(
         a.X, a.R, a.K, a.ld, a.plane_stride, a.w, a.S, dig, a.digit_ld, a.exps, status_ptr());
   }
   return cuda_fail(cudaGetLastError(), "split pieces launch");
 }
 
+// The pieces of a (b: of both operands in one launch).
+template <int MW, typename Out, int NL>
+int launch_pieces_ab(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
+  return b ? launch_pieces_pair<MW, Out, NL>(a, *b, s) : launch_pieces<MW, Out, NL>(a, s);
+}
+
 template <int MW, typename Out>
-int launch_pieces_nl(const SplitArgs &a, cudaStream_t s) {
-  const int bits = a.w * a.S + 3;  // |T| < m 2^(wS-2) < 2^(wS+1), one sign bit
-  if (bits <= 128) return launch_pieces<MW, Out, 2>(a, s);
-  if (bits <= 256) return launch_pieces<MW, Out, 4>(a, s);
-  if (bits <= 384) return launch_pieces<MW, Out, 6>(a, s);
-  if (bits <= 512) return launch_pieces<MW, Out, 8>(a, s);
-  if (bits <= 640) return launch_pieces<MW, Out, 10>(a, s);
-  return fail(MW_EUNSUPPORTED, "w*S = %d too large (at most 637 bits)", a.w * a.S);
+int launch_pieces_nl(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
+  const int S = b ? std::max(a.S, b->S) : a.S;
+  const int bits = a.w * S + 3;  // |T| < m 2^(wS-2) < 2^(wS+1), one sign bit
+  if (bits <= 128) return launch_pieces_ab<MW, Out, 2>(a, b, s);
+  if (bits <= 256) return launch_pieces_ab<MW, Out, 4>(a, b, s);
+  if (bits <= 384) return launch_pieces_ab<MW, Out, 6>(a, b, s);
+  if (bits <= 512) return launch_pieces_ab<MW, Out, 8>(a, b, s);
+  if (bits <= 640) return launch_pieces_ab<MW, Out, 10>(a, b, s);
+  return fail(MW_EUNSUPPORTED, "w*S = %d too large (at most 637 bits)", a.w * S);
 }
 
 template <typename Out>
-int launch_pieces_m(const SplitArgs &a, cudaStream_t s) {
+int launch_pieces_m(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
   switch (a.m) {
-    case 2: return launch_pieces_nl<2, Out>(a, s);
-    case 4: return launch_pieces_nl<4, Out>(a, s);
-    case 8: return launch_pieces_nl<8, Out>(a, s);
+    case 2: return launch_pieces_nl<2, Out>(a, b, s);
+    case 4: return launch_pieces_nl<4, Out>(a, b, s);
+    case 8: return launch_pieces_nl<8, Out>(a, b, s);
     case 16:
       // hexa doubles: bfloat16 pieces (MW_OZAKI) only
       if constexpr (std::is_same<Out, __nv_bfloat16>::value) {
-        const int bits = a.w * a.S + 3;
-        if (bits <= 768) return launch_pieces<16, Out, 12>(a, s);
-        if (bits <= 896) return launch_pieces<16, Out, 14>(a, s);
-        if (bits <= 1024) return launch_pieces<16, Out, 16>(a, s);
-        return fail(MW_EUNSUPPORTED, "w*S = %d too large (at most 1021 bits)", a.w * a.S);
+        const int S = b ? std::max(a.S, b->S) : a.S;
+        const int bits = a.w * S + 3;
+        if (bits <= 768) return launch_pieces_ab<16, Out, 12>(a, b, s);
+        if (bits <= 896) return launch_pieces_ab<16, Out, 14>(a, b, s);
+        if (bits <= 1024) return launch_pieces_ab<16, Out, 16>(a, b, s);
+        return fail(MW_EUNSUPPORTED, "w*S = %d too large (at most 1021 bits)", a.w * S);
       } else {
         return fail(MW_EUNSUPPORTED, "m = 16 is cut into bfloat16 pieces only");
       }
@@ -320,8 +494,39 @@ int launch_split(const SplitArgs &a, bool exponents_only, cudaStream_t s) {
   int rc = launch_exps(b, a.m, 0, nullptr, s);
   if (rc || exponents_only) return rc;
   if (a.nmod > 0) return launch_residues(b, s);
-  if (a.format == MW_DIGITS_BF16) return launch_pieces_m<__nv_bfloat16>(a, s);
-  return launch_pieces_m<double>(a, s);
+  return launch_digits(a, nullptr, s);
+}
+
+int launch_digits(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
+  if (a.format == MW_DIGITS_BF16) return launch_pieces_m<__nv_bfloat16>(a, b, s);
+  return launch_pieces_m<double>(a, b, s);
+}
+
+bool exps_together(const SplitArgs &a, const SplitArgs &b, bool exponents_only) {
+  if (a.K > kPairMaxK || (a.R + 7) / 8 + (b.R + 7) / 8 > 0x7fffffff) return false;
+  return exponents_only || a.m * (a.R + b.R) * a.K <= kPairMaxWords;
+}
+
+bool digits_together(const SplitArgs &a, const SplitArgs &b) {
+  return a.nmod == 0 && (a.R + b.R) * a.K <= kPairMaxEntries;
+}
+
+int launch_exps_pair(const SplitArgs &a, const SplitArgs &b, unsigned long long *counter,
+                     cudaStream_t s) {
+  auto args = [](const SplitArgs &x) {
+    return ExpsArgs{x.X, x.R, x.K, x.ld, x.plane_stride, x.trans, x.range,
+                    x.exps, x.spread, x.max_spread};
+  };
+  const ExpsArgs ea = args(a), eb = args(b);
+  const unsigned na = (unsigned)exps_pair_blocks(ea), nb = (unsigned)exps_pair_blocks(eb);
+  switch (a.m) {
+    case 2: exps_pair_kernel<2><<<na + nb, 256, 0, s>>>(ea, eb, na, counter, status_ptr()); break;
+    case 4: exps_pair_kernel<4><<<na + nb, 256, 0, s>>>(ea, eb, na, counter, status_ptr()); break;
+    case 8: exps_pair_kernel<8><<<na + nb, 256, 0, s>>>(ea, eb, na, counter, status_ptr()); break;
+    case 16: exps_pair_kernel<16><<<na + nb, 256, 0, s>>>(ea, eb, na, counter, status_ptr()); break;
+    default: return fail(MW_EINVAL, "m must be 2, 4, 8 or 16");
+  }
+  return cuda_fail(cudaGetLastError(), "split exponent launch");
 }
 
 }  // namespace mw
