@@ -25,6 +25,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <memory>
+#include <mutex>
+#include <new>
 #include <type_traits>
 #include <vector>
 
@@ -819,9 +822,10 @@ int launch_residues(const SplitArgs &a, cudaStream_t s) {
   return fail(MW_EUNSUPPORTED, "residue form: m = %d (2 or 4)", a.m);
 }
 
-int launch_crt_combine(const OzakiArgs &a, cudaStream_t s) {
-  const int D = a.D;
-  if (D < 1 || D > kNumModuli) return fail(MW_EINVAL, "residue form: %d moduli", D);
+namespace {
+
+// The reconstruction's constants for the first D moduli; NL in *limbs.
+int fuse_constants(int D, CrtFuse &F, int *limbs) {
   Big P{1};
   for (int t = 0; t < D; ++t) big_mul_small(P, kModuli[t]);
   int hb = 31;                                       // bit length of P: bl
@@ -831,7 +835,7 @@ int launch_crt_combine(const OzakiArgs &a, cudaStream_t s) {
   const int top = std::max(2, (bl + 2 + 31) / 32);
   const int NL = std::max(8, (top + 3) / 4 * 4);   // limbs computed (N of the MMA / 4)
   if (NL > kCrtMaxLimbs) return fail(MW_EUNSUPPORTED, "residue form: modulus product of %d bits", bl);
-  CrtFuse F{};
+  F = CrtFuse{};
   F.D = D;
   F.top = top;
   for (int t = 0; t < D; ++t) {
@@ -870,6 +874,37 @@ int launch_crt_combine(const OzakiArgs &a, cudaStream_t s) {
   for (int l = (int)P.size() - 1; l >= lo; --l) Pd = Pd * 4294967296.0 + (double)P[l];
   const int e = 32 * lo;
   for (int i = 0; i < 8; ++i) F.cz[i] = (float)std::ldexp(1.0 / Pd, 8 * (4 * top - 8 + i) - e);
+  *limbs = NL;
+  return MW_OK;
+}
+
+// They depend on D alone: computed on its first use (some 60 us of host arithmetic) and
+// kept, one entry per length of the moduli table.
+int fuse_constants_kept(int D, const CrtFuse **F, int *limbs) {
+  static std::mutex mu;
+  static std::unique_ptr<CrtFuse> kept[kNumModuli + 1];
+  static int nl[kNumModuli + 1];
+  std::lock_guard<std::mutex> lock(mu);
+  if (!kept[D]) {
+    std::unique_ptr<CrtFuse> f(new (std::nothrow) CrtFuse);
+    if (!f) return fail(MW_ECUDA, "out of host memory");
+    const int rc = fuse_constants(D, *f, &nl[D]);
+    if (rc) return rc;
+    kept[D] = std::move(f);
+  }
+  *F = kept[D].get();
+  *limbs = nl[D];
+  return MW_OK;
+}
+
+}  // namespace
+
+int launch_crt_combine(const OzakiArgs &a, cudaStream_t s) {
+  const int D = a.D;
+  if (D < 1 || D > kNumModuli) return fail(MW_EINVAL, "residue form: %d moduli", D);
+  const CrtFuse *F = nullptr;
+  int NL = 0, rc = fuse_constants_kept(D, &F, &NL);
+  if (rc) return rc;
   // residues: bf16 planes [t][i][j], rows of crt_ld(N); boxes of 64 outputs of
   // one row x every modulus (moduli past D, outputs past N: zeros)
   alignas(64) CUtensorMap map;
@@ -877,11 +912,11 @@ int launch_crt_combine(const OzakiArgs &a, cudaStream_t s) {
   const uint64_t dims[3] = {(uint64_t)a.N, (uint64_t)a.M, (uint64_t)D};
   const uint64_t strides[2] = {(uint64_t)ld * 2, (uint64_t)a.M * ld * 2};
   const uint32_t box[3] = {64, 1, (uint32_t)((D + 15) & ~15)};
-  int rc = make_map_bf16(&map, a.partials, 3, dims, strides, box);
+  rc = make_map_bf16(&map, a.partials, 3, dims, strides, box);
   if (rc) return rc;
   switch (a.m) {
-    case 2: return launch_crt_fuse_m<2>(a, F, NL, map, s);
-    case 4: return launch_crt_fuse_m<4>(a, F, NL, map, s);
+    case 2: return launch_crt_fuse_m<2>(a, *F, NL, map, s);
+    case 4: return launch_crt_fuse_m<4>(a, *F, NL, map, s);
   }
   return fail(MW_EUNSUPPORTED, "residue form: m = %d (2 or 4)", a.m);
 }

@@ -164,12 +164,12 @@ struct Maps {
   CUtensorMap a[NBOX], b[NBOXB], out;
 };
 __host__ __device__ constexpr int box_rows(int i) { return 16 * (i + 1); }
-__device__ __forceinline__ int box_index(int64_t rows) {
+__host__ __device__ __forceinline__ int box_index(int64_t rows) {
   return rows <= 16 ? 0 : rows >= 256 ? NBOX - 1 : (int)((rows + 15) >> 4) - 1;
 }
 // B boxes in steps of 8 rows: a stacked block of N8 rows starts on a swizzle atom
 __host__ __device__ constexpr int box_rows_b(int i) { return 8 * (i + 1); }
-__device__ __forceinline__ int box_index_b(int64_t rows) {
+__host__ __device__ __forceinline__ int box_index_b(int64_t rows) {
   return rows <= 8 ? 0 : rows >= 256 ? NBOXB - 1 : (int)((rows + 7) >> 3) - 1;
 }
 
@@ -770,10 +770,28 @@ int launch_product(const ProductLaunch &a, cudaStream_t s) {
       std::swap(P.gorder[j], P.gorder[j - 1]);
   Maps maps;
   int rc = MW_OK;
-  for (int i = 0; i < NBOX && !rc; ++i)
-    rc = make_map_2d(&maps.a[i], a.pieceA, a.Kpitch, a.rowsA, std::min(box_rows(i), BM));
-  for (int i = 0; i < NBOXB && !rc; ++i)
-    rc = make_map_2d(&maps.b[i], a.pieceB, a.KpitchB, a.rowsB, std::min(box_rows_b(i), bn));
+  if (a.info) {
+    for (int i = 0; i < NBOX && !rc; ++i)
+      rc = make_map_2d(&maps.a[i], a.pieceA, a.Kpitch, a.rowsA, std::min(box_rows(i), BM));
+    for (int i = 0; i < NBOXB && !rc; ++i)
+      rc = make_map_2d(&maps.b[i], a.pieceB, a.KpitchB, a.rowsB, std::min(box_rows_b(i), bn));
+  } else {
+    // a single product has full tiles and one ragged tile each way: two maps an operand
+    // are encoded, the others are copies (never used; the kernel prefetches every
+    // entry).  Encoding all 48 cost a call about 5 us on the host.
+    const int fa = box_index(std::min<int64_t>(a.M, BM)), fb = box_index_b(std::min<int64_t>(a.N, bn));
+    const int la = a.M % BM ? box_index(a.M % BM) : fa, lb = a.N % bn ? box_index_b(a.N % bn) : fb;
+    rc = make_map_2d(&maps.a[fa], a.pieceA, a.Kpitch, a.rowsA, std::min(box_rows(fa), BM));
+    if (!rc) rc = make_map_2d(&maps.b[fb], a.pieceB, a.KpitchB, a.rowsB, std::min(box_rows_b(fb), bn));
+    for (int i = 0; i < NBOX; ++i)
+      if (i != fa) maps.a[i] = maps.a[fa];
+    for (int i = 0; i < NBOXB; ++i)
+      if (i != fb) maps.b[i] = maps.b[fb];
+    if (!rc && la != fa)
+      rc = make_map_2d(&maps.a[la], a.pieceA, a.Kpitch, a.rowsA, std::min(box_rows(la), BM));
+    if (!rc && lb != fb)
+      rc = make_map_2d(&maps.b[lb], a.pieceB, a.KpitchB, a.rowsB, std::min(box_rows_b(lb), bn));
+  }
   if (!rc && a.crt && bn == 256) {
     // residue planes [t][i][j], rows of crt_ld(N) elements
     const uint64_t ld = (uint64_t)crt_ld(a.N);
