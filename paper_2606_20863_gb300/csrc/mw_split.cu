@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(256)
 // Pieces of both operands in one launch, for small products (kPairMaxEntries), where
 // a second stream's fork and join cost more than the kernels beside each other save:
 // with the exponents together 64^3 double doubles 45.6 -> 31.9 us a call (37 -> 25
-// replayed from a graph), 64^3 octo doubles 82.7 -> 66.3.
+// replayed from a graph).
 constexpr int64_t kPairMaxEntries = 1 << 18;
 template <typename Out> struct PieceArgs {
   const double *X;
@@ -401,10 +401,14 @@ int launch_pieces(const SplitArgs &a, cudaStream_t s) {
   return cuda_fail(cudaGetLastError(), "split pieces launch");
 }
 
-// The pieces of a (b: of both operands in one launch).
+// The pieces of a (b: of both operands, on one stream).
 template <int MW, typename Out, int NL>
 int launch_pieces_ab(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
-  return b ? launch_pieces_pair<MW, Out, NL>(a, *b, s) : launch_pieces<MW, Out, NL>(a, s);
+  if (!b) return launch_pieces<MW, Out, NL>(a, s);
+  // wider entries: two launches (their kernels take minutes to compile twice)
+  if constexpr (NL <= 4) return launch_pieces_pair<MW, Out, NL>(a, *b, s);
+  const int rc = launch_pieces<MW, Out, NL>(a, s);
+  return rc ? rc : launch_pieces<MW, Out, NL>(*b, s);
 }
 
 template <int MW, typename Out>
