@@ -661,13 +661,9 @@ int launch_split_w(const BInfo *info, const BHeader *hdr, const mw_batch &b, con
   // the 16-row tile, then (w = 8, m >= 8) 256 columns of (64 NL - 8) / 24 + 4 slots
   const size_t sm = (size_t)MW * 16 * 33 * sizeof(double) +
                     (W8 && MW >= 8 ? (size_t)((64 * NL - 8) / 24 + 4) * 256 * sizeof(uint32_t) : 0);
-  static bool attr_set = false;  // once per instantiation
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(batch_split_cols_kernel<MW, NL, W8>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return cuda_fail(e, "batched split smem attribute");
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> granted{0};
+  cudaError_t e = allow_smem(granted, batch_split_cols_kernel<MW, NL, W8>, sm);
+  if (e != cudaSuccess) return cuda_fail(e, "batched split smem attribute");
   batch_split_cols_kernel<MW, NL, W8><<<grid_for(2), 256, sm, s>>>(
       info, hdr, b.count, p.w, p.S_B, L.KpitchB, reinterpret_cast<__nv_bfloat16 *>(w8 + L.pieceB),
       reinterpret_cast<int32_t *>(w8 + L.eB), reinterpret_cast<int32_t *>(w8 + L.spB),

@@ -452,22 +452,21 @@ int launch_residues_t(const SplitArgs &a, cudaStream_t s) {
   if (rc) return rc;
   const size_t smem = residue_smem(npad);
   auto kern = a.trans ? residues_mma_kernel<MW, NL, true> : residues_mma_kernel<MW, NL, false>;
-  static bool attr[2] = {false, false};
-  if (!attr[a.trans ? 1 : 0]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)residue_smem(96));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                               cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return cuda_fail(e, "residue split smem attribute");
-    attr[a.trans ? 1 : 0] = true;
-  }
+  static std::atomic<uint64_t> granted[2];
+  cudaError_t e = once_a_device(granted[a.trans ? 1 : 0], [&] {
+    const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)residue_smem(96));
+    return r != cudaSuccess ? r
+                            : cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                   cudaSharedmemCarveoutMaxShared);
+  });
+  if (e != cudaSuccess) return cuda_fail(e, "residue split smem attribute");
   int dev = 0, nsm = 0, smem_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+  e = cudaFuncGetAttributes(&fa, kern);
   if (e != cudaSuccess) return cuda_fail(e, "residue split attributes");
   // resident CTAs: shared memory (1 KB reserved per CTA), registers, tensor memory
   const int by_smem = smem_sm / (int)(smem + 1024);
@@ -721,24 +720,23 @@ int launch_crt_fuse_t(const OzakiArgs &a, const CrtFuse &F, const CUtensorMap &m
   const size_t smem = fuse_smem(F.D, NL);
   if (2 * NL > ((F.D + 15) & ~15))                 // a buffer holds the limb columns
     return fail(MW_EUNSUPPORTED, "residue form: %d limbs of %d moduli", NL, F.D);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(crt_fuse_kernel<MW, NL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)fuse_smem(kCrtMaxModuli, NL));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(crt_fuse_kernel<MW, NL>,
-                               cudaFuncAttributePreferredSharedMemoryCarveout,
-                               cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return cuda_fail(e, "reconstruction smem attribute");
-    attr = true;
-  }
+  static std::atomic<uint64_t> granted{0};
+  cudaError_t e = once_a_device(granted, [] {
+    const cudaError_t r = cudaFuncSetAttribute(crt_fuse_kernel<MW, NL>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)fuse_smem(kCrtMaxModuli, NL));
+    return r != cudaSuccess ? r
+                            : cudaFuncSetAttribute(crt_fuse_kernel<MW, NL>,
+                                                   cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                   cudaSharedmemCarveoutMaxShared);
+  });
+  if (e != cudaSuccess) return cuda_fail(e, "reconstruction smem attribute");
   int dev = 0, nsm = 0, smem_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, crt_fuse_kernel<MW, NL>);
+  e = cudaFuncGetAttributes(&fa, crt_fuse_kernel<MW, NL>);
   if (e != cudaSuccess) return cuda_fail(e, "reconstruction attributes");
   // resident CTAs: shared memory (1 KB reserved per CTA), registers, tensor memory
   const int per_sm = std::max(1, std::min({smem_sm / (int)(smem + 1024),

@@ -309,13 +309,9 @@ int launch_dot_s(const DotArgs &a, cudaStream_t st) {
   constexpr size_t smem = MW >= 8 ? 2 * 2 * MW * kDotThreads * sizeof(double) +
                                         (size_t)(S + 3) * kDotThreads * sizeof(uint32_t)
                                   : 0;
-  static bool attr_set = false;   // once per instance
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(dot_kernel<MW, S, NLF>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "dot kernel smem attribute");
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> granted{0};
+  cudaError_t e = allow_smem(granted, dot_kernel<MW, S, NLF>, smem);
+  if (e != cudaSuccess) return cuda_fail(e, "dot kernel smem attribute");
   dot_kernel<MW, S, NLF><<<grid, kDotThreads, smem, st>>>(a);
   return cuda_fail(cudaGetLastError(), "dot kernel launch");
 }

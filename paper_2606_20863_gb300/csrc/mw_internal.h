@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <functional>
 
 #include "../../include/mw.h"
@@ -16,6 +17,25 @@ int cuda_fail(cudaError_t e, const char *what);
 
 // Device address of the status word of the current device.
 unsigned int *status_ptr();
+
+// A kernel's attributes (its limit of dynamic shared memory) hold for one device at a
+// time: set() runs on the first call with each device current, done keeps a bit a device.
+template <class F> cudaError_t once_a_device(std::atomic<uint64_t> &done, F set) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0;     // past 64 devices: set on every call
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = set();
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
+// The same for the limit alone.
+template <class K> cudaError_t allow_smem(std::atomic<uint64_t> &done, K *kernel, size_t bytes) {
+  return once_a_device(done, [&] {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
+}
 
 inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 

@@ -803,36 +803,24 @@ int launch_product(const ProductLaunch &a, cudaStream_t s) {
     memset(&maps.out, 0, sizeof maps.out);
   }
   if (rc) return rc;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(ozaki_kernel<128, true, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Shape<128, true>::SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ozaki_kernel<128, false, false>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)Shape<128, false>::SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ozaki_kernel<256, true, false>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)Shape<256, true>::SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ozaki_kernel<256, true, true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)Shape<256, true>::SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ozaki_kernel<256, true, false, true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kernel_smem<256, true, true>());
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ozaki_kernel<128, true, false, true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)Shape<128, true>::SMEM);
-    if (e != cudaSuccess) return cuda_fail(e, "product kernel smem attribute");
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> granted{0};
+  cudaError_t e = once_a_device(granted, [] {
+    cudaError_t r = cudaSuccess;
+    auto allow = [&](auto *kernel, size_t bytes) {
+      if (r == cudaSuccess)
+        r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    allow(ozaki_kernel<128, true, false>, Shape<128, true>::SMEM);
+    allow(ozaki_kernel<128, false, false>, Shape<128, false>::SMEM);
+    allow(ozaki_kernel<256, true, false>, Shape<256, true>::SMEM);
+    allow(ozaki_kernel<256, true, true>, Shape<256, true>::SMEM);
+    allow(ozaki_kernel<256, true, false, true>, kernel_smem<256, true, true>());
+    allow(ozaki_kernel<128, true, false, true>, Shape<128, true>::SMEM);
+    return r;
+  });
+  if (e != cudaSuccess) return cuda_fail(e, "product kernel smem attribute");
   if (!a.counter_clear) {
-    cudaError_t e = cudaMemsetAsync(a.next_item, 0, sizeof(unsigned long long), s);
+    e = cudaMemsetAsync(a.next_item, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return cuda_fail(e, "work counter reset");
   }
   int dev = 0, nsm = 0;

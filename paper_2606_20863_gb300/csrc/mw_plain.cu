@@ -220,13 +220,9 @@ int launch(const PlainArgs &a, cudaStream_t s) {
   const size_t smem = plain_split_smem(a.S_A, a.S_B, a.D, KC);
   const int64_t tiles = (a.N + SC - 1) / SC * ((a.M + SR - 1) / SR);
   if (smem <= 232448 && tiles <= 0x7fffffff) {
-    static bool attr_set = false;   // once per instance
-    if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(plain_split_kernel<MW>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-      if (e != cudaSuccess) return cuda_fail(e, "plain kernel smem attribute");
-      attr_set = true;
-    }
+    static std::atomic<uint64_t> granted{0};
+    cudaError_t e = allow_smem(granted, plain_split_kernel<MW>, 232448);
+    if (e != cudaSuccess) return cuda_fail(e, "plain kernel smem attribute");
     plain_split_kernel<MW><<<(unsigned)tiles, 32 * SWARPS, smem, s>>>(a, KC);
     return cuda_fail(cudaGetLastError(), "plain kernel launch");
   }

@@ -271,14 +271,9 @@ __global__ void __launch_bounds__(32 * kSeriesWarps, MW == 16 ? 1 : 2)
 
 template <int MW, int S>
 int launch_series_s(const DotArgs &a, cudaStream_t st) {
-  static bool attr_set = false;   // once per instance
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(series_kernel<MW, S>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSeriesSmem);
-    if (e != cudaSuccess) return cuda_fail(e, "series kernel smem attribute");
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> granted{0};
+  cudaError_t e = allow_smem(granted, series_kernel<MW, S>, kSeriesSmem);
+  if (e != cudaSuccess) return cuda_fail(e, "series kernel smem attribute");
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);

@@ -364,14 +364,9 @@ int launch_pieces_pair(const SplitArgs &a, const SplitArgs &b, cudaStream_t s) {
                               : (x.R * (x.digit_ld / 2) + 255) / 256);
   };
   const size_t sm = a.trans || b.trans ? (size_t)MW * 32 * 33 * sizeof(double) : 0;
-  static bool attr_set = false;  // once per instantiation
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(pieces_pair_kernel<MW, NL, Out>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         MW * 32 * 33 * (int)sizeof(double));
-    if (e != cudaSuccess) return cuda_fail(e, "split smem attribute");
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> granted{0};
+  cudaError_t e = allow_smem(granted, pieces_pair_kernel<MW, NL, Out>, MW * 32 * 33 * sizeof(double));
+  if (e != cudaSuccess) return cuda_fail(e, "split smem attribute");
   pieces_pair_kernel<MW, NL, Out><<<blocks(a) + blocks(b), 256, sm, s>>>(args(a), args(b), blocks(a),
                                                                         a.w, status_ptr());
   return cuda_fail(cudaGetLastError(), "split pieces launch");
@@ -388,13 +383,9 @@ int launch_pieces(const SplitArgs &a, cudaStream_t s) {
   } else {
     dim3 grid((unsigned)((a.R + 31) / 32), (unsigned)((a.digit_ld + 31) / 32));
     const size_t sm = (size_t)MW * 32 * 33 * sizeof(double);
-    static bool attr_set = false;  // once per instantiation
-    if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(pieces_cols_kernel<MW, NL, Out>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return cuda_fail(e, "split smem attribute");
-      attr_set = true;
-    }
+    static std::atomic<uint64_t> granted{0};
+    cudaError_t e = allow_smem(granted, pieces_cols_kernel<MW, NL, Out>, sm);
+    if (e != cudaSuccess) return cuda_fail(e, "split smem attribute");
     pieces_cols_kernel<MW, NL, Out><<<grid, 256, sm, s>>>(
         a.X, a.R, a.K, a.ld, a.plane_stride, a.w, a.S, dig, a.digit_ld, a.exps, status_ptr());
   }
