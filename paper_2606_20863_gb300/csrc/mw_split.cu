@@ -327,8 +327,14 @@ __global__ void __launch_bounds__(256)
 // Pieces of both operands in one launch, for small products (kPairMaxEntries), where
 // a second stream's fork and join cost more than the kernels beside each other save:
 // with the exponents together 64^3 double doubles 45.6 -> 31.9 us a call (37 -> 25
-// replayed from a graph).
+// replayed from a graph).  Only for entries of up to kPairMaxBits bits: the wider
+// kernels take minutes to compile twice, and their two launches belong beside each
+// other on two streams (64^3, one after the other / beside each other: octo doubles
+// 77 / 67 us, hexa doubles 237 / 194, 50-bit spreads of quad doubles 53 / 50; 32 x 32 x
+// 512 hexa doubles with A transposed 728 / 628; equal from 256^3 on).
 constexpr int64_t kPairMaxEntries = 1 << 18;
+constexpr int kPairMaxBits = 256;
+inline int piece_bits(int w, int S) { return w * S + 3; }   // |T| < m 2^(wS-2) < 2^(wS+1), one sign bit
 template <typename Out> struct PieceArgs {
   const double *X;
   int64_t R, K, ld, ps, dld;
@@ -392,20 +398,18 @@ int launch_pieces(const SplitArgs &a, cudaStream_t s) {
   return cuda_fail(cudaGetLastError(), "split pieces launch");
 }
 
-// The pieces of a (b: of both operands, on one stream).
+// The pieces of a (b: of both operands, of at most kPairMaxBits bits).
 template <int MW, typename Out, int NL>
 int launch_pieces_ab(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
   if (!b) return launch_pieces<MW, Out, NL>(a, s);
-  // wider entries: two launches (their kernels take minutes to compile twice)
-  if constexpr (NL <= 4) return launch_pieces_pair<MW, Out, NL>(a, *b, s);
-  const int rc = launch_pieces<MW, Out, NL>(a, s);
-  return rc ? rc : launch_pieces<MW, Out, NL>(*b, s);
+  if constexpr (64 * NL <= kPairMaxBits) return launch_pieces_pair<MW, Out, NL>(a, *b, s);
+  return fail(MW_EUNSUPPORTED, "pieces of both operands in one launch: %d limbs", NL);
 }
 
 template <int MW, typename Out>
 int launch_pieces_nl(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
   const int S = b ? std::max(a.S, b->S) : a.S;
-  const int bits = a.w * S + 3;  // |T| < m 2^(wS-2) < 2^(wS+1), one sign bit
+  const int bits = piece_bits(a.w, S);
   if (bits <= 128) return launch_pieces_ab<MW, Out, 2>(a, b, s);
   if (bits <= 256) return launch_pieces_ab<MW, Out, 4>(a, b, s);
   if (bits <= 384) return launch_pieces_ab<MW, Out, 6>(a, b, s);
@@ -424,7 +428,7 @@ int launch_pieces_m(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
       // hexa doubles: bfloat16 pieces (MW_OZAKI) only
       if constexpr (std::is_same<Out, __nv_bfloat16>::value) {
         const int S = b ? std::max(a.S, b->S) : a.S;
-        const int bits = a.w * S + 3;
+        const int bits = piece_bits(a.w, S);
         if (bits <= 768) return launch_pieces_ab<16, Out, 12>(a, b, s);
         if (bits <= 896) return launch_pieces_ab<16, Out, 14>(a, b, s);
         if (bits <= 1024) return launch_pieces_ab<16, Out, 16>(a, b, s);
@@ -503,7 +507,8 @@ bool exps_together(const SplitArgs &a, const SplitArgs &b, bool exponents_only) 
 }
 
 bool digits_together(const SplitArgs &a, const SplitArgs &b) {
-  return a.nmod == 0 && (a.R + b.R) * a.K <= kPairMaxEntries;
+  return a.nmod == 0 && (a.R + b.R) * a.K <= kPairMaxEntries &&
+         piece_bits(a.w, std::max(a.S, b.S)) <= kPairMaxBits;
 }
 
 int launch_exps_pair(const SplitArgs &a, const SplitArgs &b, unsigned long long *counter,

@@ -1,0 +1,29 @@
+"""Where the pieces of a small product's two operands are cut: in one launch for entries
+of up to 256 bits, beside each other on two streams for wider ones.  The library's host
+code on a stand-in runtime; no GPU."""
+import pytest
+
+import host_runtime
+
+
+@pytest.fixture(scope="module")
+def host(mw, tmp_path_factory):
+    lib = host_runtime.link(mw, str(tmp_path_factory.mktemp("host")))
+    if lib is None:
+        pytest.skip("no C++ compiler")
+    return lib
+
+
+@pytest.mark.parametrize("m,range_,M,N,K,ta,tb,together", [
+    (2, 4, 64, 64, 64, 0, 0, True), (4, 4, 64, 64, 64, 1, 0, True), (4, 4, 1, 1, 1, 0, 0, True),
+    (4, 60, 64, 64, 64, 0, 0, False), (8, 4, 64, 64, 64, 0, 0, False),
+    (8, 4, 8, 8, 8, 1, 1, False), (16, 4, 32, 32, 512, 1, 0, False), (16, 4, 64, 64, 64, 0, 1, False),
+])
+def test_wide_entries_on_two_streams(host, m, range_, M, N, K, ta, tb, together):
+    p = host.plan(m, "ozaki", M, N, K, range_, range_)
+    ls = host.launches(lambda: host.gemm(p, M, N, K, ta, tb))
+    cuts = [l for l in ls if "pieces_" in l[0]]
+    if together:
+        assert len(cuts) == 1 and "pieces_pair" in cuts[0][0] and cuts[0][4] == 0
+    else:
+        assert len(cuts) == 2 and cuts[0][4] == 0 and cuts[1][4] != 0
