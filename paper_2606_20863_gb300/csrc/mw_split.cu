@@ -144,14 +144,28 @@ __global__ void exps_finalize_kernel(int64_t R, int *E, int *spread, int *max_sp
 // Pass 1 of both operands of a product in one launch: no atomics on the rows, no
 // clearing, no finalize, no second stream.  trans = 0: a warp per row, eight rows a
 // block; trans = 1: 8 columns x 32 rows of the stored matrix at a time; either way
-// the threads that see a row or column see all of it, so reductions are short
-// (kPairMaxK) and, in a product, operands small (kPairMaxWords: 384^3 quad doubles 120
-// -> 114 us, 512^3 149 -> 159, 256^3 octo doubles 150 -> 137, 384^3 236 -> 246; above
-// that the two-stream passes over chunks keep more loads in flight).  The spread
-// measurement, which waits for the result, always takes it (2048 x 1024 double
-// doubles: 96 -> 46 us a call).  The first block clears the product kernel's work
-// counter.
-constexpr int64_t kPairMaxK = 2048;
+// the threads that see a row or column see all of it, one entry in 32 each, so
+// reductions are short (pair_max_k) and, in a product, operands small (kPairMaxWords:
+// 384^3 quad doubles 120 -> 114 us, 512^3 149 -> 159, 256^3 octo doubles 150 -> 137,
+// 384^3 236 -> 246; above that the two-stream passes over chunks keep more loads in
+// flight).  The limits on the reduction, us a call apart / together, 32 x 32 outputs:
+//   products   m = 2  K = 1,024  106 / 99   2,048  170 / 172 (128 x 128: 176 / 181)
+//              m = 4  K = 1,024  172 / 170  2,048  299 / 310 (residues: 63 / 61, 78 / 88)
+//              m = 8  K = 512    190 / 183  1,024  313 / 315  2,048  568 / 588
+//              m = 16 K = 512    643 / 630  1,024  1,130 / 1,126
+//   the spread measurement (16 to 1,024 rows), which waits for the result:
+//              m = 2  K = 2,048  53 / 48    m = 4  1,024  56 / 47, 2,048  58 / 59
+//              m = 8  K = 1,024  61 / 58, 2,048  61 / 71
+//              m = 16 K = 1,024  62 / 57 (1,000 + 1,000 rows: 150 / 109), 2,048  62 / 72
+// Many rows (more than kPairMaxRows): a warp a short row, or eight columns of few rows,
+// leaves loads unused: 2^19 columns of 1..16 double doubles 84-125 / 117-158, of 64
+// 281 / 234; 2^19 rows of 2 580 / 172, of 128 773 / 730, of 256 872 / 1,055.
+// The first block clears the product kernel's work counter.
+inline int64_t pair_max_k(int m, bool exponents_only) {
+  if (m <= 2) return exponents_only ? 2048 : 1536;
+  return m <= 4 || exponents_only ? 1024 : 512;
+}
+constexpr int64_t kPairMaxRows = 1 << 17;
 constexpr int64_t kPairMaxWords = 3 << 19;
 constexpr int kPairCols = 8;
 struct ExpsArgs {
@@ -502,7 +516,12 @@ int launch_digits(const SplitArgs &a, const SplitArgs *b, cudaStream_t s) {
 }
 
 bool exps_together(const SplitArgs &a, const SplitArgs &b, bool exponents_only) {
-  if (a.K > kPairMaxK || (a.R + 7) / 8 + (b.R + 7) / 8 > 0x7fffffff) return false;
+  auto few_rows = [](const SplitArgs &x) {
+    return x.R <= kPairMaxRows || (x.trans ? x.K >= 64 : x.K <= 128);
+  };
+  if (a.K > pair_max_k(a.m, exponents_only) || !few_rows(a) || !few_rows(b) ||
+      (a.R + 7) / 8 + (b.R + 7) / 8 > 0x7fffffff)
+    return false;
   return exponents_only || a.m * (a.R + b.R) * a.K <= kPairMaxWords;
 }
 
