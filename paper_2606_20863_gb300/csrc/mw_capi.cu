@@ -443,7 +443,9 @@ int split_both(const mw_plan &p, int transA, int transB, int64_t M, int64_t N, i
   // residue splits hold tensor memory on every SM they run on: with more than
   // 64 moduli two of them would not fit side by side, so they run one after the
   // other on the caller's stream
-  cudaStream_t s2 = (p.mode == MW_CRT && !exps_only && p.D > 64) ? nullptr : side_stream();
+  const bool in_a_row = (p.mode == MW_CRT && !exps_only && p.D > 64) ||
+                        (together && digits_in_a_row(a, b));
+  cudaStream_t s2 = in_a_row ? nullptr : side_stream();
   cudaEvent_t ev[2] = {nullptr, nullptr};
   bool fork = s2 != nullptr &&
               cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) == cudaSuccess &&

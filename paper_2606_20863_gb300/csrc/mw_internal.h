@@ -60,6 +60,9 @@ int launch_split(const SplitArgs &a, bool exponents_only, cudaStream_t s);
 // whether their digits are cut in one.
 bool exps_together(const SplitArgs &a, const SplitArgs &b, bool exponents_only);
 bool digits_together(const SplitArgs &a, const SplitArgs &b);
+// Otherwise, with the exponents in one launch: whether the two cuts go one after the
+// other on the caller's stream instead of beside each other.
+bool digits_in_a_row(const SplitArgs &a, const SplitArgs &b);
 int launch_exps_pair(const SplitArgs &a, const SplitArgs &b, unsigned long long *counter,
                      cudaStream_t s);
 // Pieces of a (and of *b unless NULL, in the same launch) from their exponents.

@@ -345,9 +345,14 @@ __global__ void __launch_bounds__(256)
 // kernels take minutes to compile twice, and their two launches belong beside each
 // other on two streams (64^3, one after the other / beside each other: octo doubles
 // 77 / 67 us, hexa doubles 237 / 194, 50-bit spreads of quad doubles 53 / 50; 32 x 32 x
-// 512 hexa doubles with A transposed 728 / 628; equal from 256^3 on).
+// 512 hexa doubles with A transposed 728 / 628).  One after the other again from
+// kRowMinEntries on when A and B are as stored (k contiguous in A only), where each
+// kernel fills the GPU: 290^3 quad doubles of wide spread 106 / 112, 300^3 octo doubles
+// 178 / 184, equal at 256^3; with a transpose beside each other stays faster (98-100 /
+// 106-107, 159-170 / 169-182).
 constexpr int64_t kPairMaxEntries = 1 << 18;
 constexpr int kPairMaxBits = 256;
+constexpr int64_t kRowMinEntries = 1 << 17;
 inline int piece_bits(int w, int S) { return w * S + 3; }   // |T| < m 2^(wS-2) < 2^(wS+1), one sign bit
 template <typename Out> struct PieceArgs {
   const double *X;
@@ -528,6 +533,11 @@ bool exps_together(const SplitArgs &a, const SplitArgs &b, bool exponents_only) 
 bool digits_together(const SplitArgs &a, const SplitArgs &b) {
   return a.nmod == 0 && (a.R + b.R) * a.K <= kPairMaxEntries &&
          piece_bits(a.w, std::max(a.S, b.S)) <= kPairMaxBits;
+}
+
+bool digits_in_a_row(const SplitArgs &a, const SplitArgs &b) {
+  const int64_t entries = (a.R + b.R) * a.K;
+  return a.nmod == 0 && entries > kRowMinEntries && entries <= kPairMaxEntries && !a.trans && b.trans;
 }
 
 int launch_exps_pair(const SplitArgs &a, const SplitArgs &b, unsigned long long *counter,

@@ -1,6 +1,7 @@
 """Where the pieces of a small product's two operands are cut: in one launch for entries
-of up to 256 bits, beside each other on two streams for wider ones.  The library's host
-code on a stand-in runtime; no GPU."""
+of up to 256 bits, beside each other on two streams for wider ones (one after the other
+where the operands as stored fill the GPU each).  The library's host code on a stand-in
+runtime; no GPU."""
 import pytest
 
 import host_runtime
@@ -27,3 +28,14 @@ def test_wide_entries_on_two_streams(host, m, range_, M, N, K, ta, tb, together)
         assert len(cuts) == 1 and "pieces_pair" in cuts[0][0] and cuts[0][4] == 0
     else:
         assert len(cuts) == 2 and cuts[0][4] == 0 and cuts[1][4] != 0
+
+
+@pytest.mark.parametrize("m,range_,n,ta,tb,two", [
+    (4, 60, 256, 0, 0, True), (4, 60, 290, 0, 0, False), (4, 60, 362, 0, 0, False),
+    (4, 60, 363, 0, 0, True), (4, 60, 290, 1, 0, True), (4, 60, 290, 0, 1, True),
+    (8, 4, 300, 0, 0, False), (8, 4, 300, 1, 1, True),
+])
+def test_wide_entries_that_fill_the_gpu(host, m, range_, n, ta, tb, two):
+    p = host.plan(m, "ozaki", n, n, n, range_, range_)
+    cuts = [l for l in host.launches(lambda: host.gemm(p, n, n, n, ta, tb)) if "pieces_" in l[0]]
+    assert len(cuts) == 2 and (cuts[1][4] != 0) == two
