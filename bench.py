@@ -999,10 +999,12 @@ ELEMENTWISE_FP64_OPS = {2: {"add": 20, "mul": 9, "div": 79},
                         8: {"add": 552, "mul": 3655, "div": 35225}}
 # The FP64 instructions mw_elementwise issues for them: two_sum 3 (operands ordered
 # on the integer units), sums only in the last sweep of a renormalisation, no
-# products with the zero words of a quotient word.  What its roofline counts.
-ELEMENTWISE_GPU_FP64 = {2: {"add": 14, "mul": 9, "div": 52},
-                        4: {"add": 58, "mul": 231, "div": 601},
-                        8: {"add": 260, "mul": 1725, "div": 5075}}
+# products with the zero words of a quotient word, of the last remainder only the
+# leading word.  What its roofline counts (recounted in
+# tests/test_elementwise_gpu_counts.py).
+ELEMENTWISE_GPU_FP64 = {2: {"add": 14, "mul": 9, "div": 50},
+                        4: {"add": 58, "mul": 231, "div": 586},
+                        8: {"add": 260, "mul": 1725, "div": 4998}}
 
 
 def run_elementwise(args, mw, torch, dist, rank, world, dev):
