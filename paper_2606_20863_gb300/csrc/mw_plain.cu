@@ -14,9 +14,11 @@
 //
 // Tiling: a block of 16 x 16 threads computes a (16 TH) x (16 TH) tile of C,
 // thread (ty, tx) the outputs (ty + 16 a, tx + 16 b); pieces are staged in
-// shared memory 16 columns of the reduction at a time.  This kernel takes any
-// plan; plain_split_kernel below (4 x 8 outputs a CTA) is faster at every size and
-// takes the plans whose pieces fit in its shared memory.
+// shared memory 16 columns of the reduction at a time.  This kernel takes any plan;
+// plain_split_kernel below (4 x 8 outputs a CTA) takes the plans whose pieces fit in
+// its shared memory where it is the faster one (split_clocks, tile_clocks).
+#include <algorithm>
+
 #include "mw_device.cuh"
 #include "mw_eft.cuh"
 
@@ -147,10 +149,31 @@ __global__ void __launch_bounds__(256, 1) plain_kernel(PlainArgs a) {
 // rows KC + 2 apart: lanes read distinct banks or the same word).  Every partial
 // diagonal sum is exact, so the warps' sums add up to the same s_t in any order;
 // warp 0 then adds the s_t into the m-double accumulator, t in order, as
-// plain_kernel does.  plain_kernel against this one, us (FP64 floor): dd 64^3
-// 1,520 / 47 (9), dd 384^3 10,290 / 2,530 (2,420), qd 640^3 37,390 / 33,080
+// plain_kernel does.  plain_kernel against this one, us (FP64 floor), the call: dd 64^3
+// 1,400 / 36 (9), dd 384^3 10,290 / 2,530 (2,420), qd 640^3 37,390 / 33,080
 // (32,770), od 256^3 17,380 / 8,010 (6,930).
 constexpr int SR = 4, SC = 8, SWARPS = 8;
+
+// Where plain_kernel is the faster one: many tiles for the SMs and a chunk that a warp's
+// share of k (every eighth) does not divide into fours, or so many pieces that one CTA
+// fills an SM.  Clocks of an SM per pair of pieces, both kernels at two multiply-adds a
+// clock: plain_kernel pays whole rounds of tiles and k in sixteens; this kernel the share
+// of the rate that chunks of 8, 16, .. 64 columns reach (measured), 0.6 of it with one CTA
+// an SM.  us, plain_kernel / this one: qd 512 x 512 x 64 2,304 / 2,761 (S = 10, chunks of 48
+// and 16), qd 512 x 512 x 300 10,300 / 11,150, w = 8 (S = 27) 14,310 / 21,580, w = 5 (S = 44)
+// 35,300 / 62,670, od w = 16 1024 x 1024 x 40 39,430 / 54,070.  Of 240 plans and sizes
+// the rule took the slower kernel for four, 3-6 % slower (K = 40, 1,024 tiles).
+inline double tile_clocks(const PlainArgs &a, int BT, int nsm) {
+  const int64_t tiles = (a.M + BT - 1) / BT * ((a.N + BT - 1) / BT);
+  return 0.5 * BT * BT * (double)((tiles + nsm - 1) / nsm * ((a.K + 15) / 16 * 16));
+}
+inline double split_clocks(const PlainArgs &a, int KC, size_t smem, int64_t tiles, int nsm) {
+  static const double rate[] = {0.79, 0.57, 0.88, 0.92, 0.85, 0.80, 0.88, 0.96};   // by columns / 8
+  const int64_t full = a.K / KC, rest = (a.K % KC + 7) / 8;
+  const double columns = (double)full * KC / rate[KC / 8 - 1] + (rest ? 8.0 * rest / rate[rest - 1] : 0.0);
+  const double one_cta = 2 * (smem + 1024) > 233472 ? 0.6 : 1.0;
+  return 0.5 * SR * SC * std::max((double)tiles / nsm, 1.0) * columns / one_cta;
+}
 
 inline size_t plain_split_smem(int S_A, int S_B, int D, int KC) {
   return 8 * ((size_t)(SR * S_A + SC * S_B) * (KC + 2) + (size_t)SWARPS * D * 32);
@@ -219,14 +242,19 @@ int launch(const PlainArgs &a, cudaStream_t s) {
   while (KC > 8 && plain_split_smem(a.S_A, a.S_B, a.D, KC) > 115712) KC -= 8;
   const size_t smem = plain_split_smem(a.S_A, a.S_B, a.D, KC);
   const int64_t tiles = (a.N + SC - 1) / SC * ((a.M + SR - 1) / SR);
-  if (smem <= 232448 && tiles <= 0x7fffffff) {
+  constexpr int BT = 16 * TH;
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (smem <= 232448 && tiles <= 0x7fffffff &&
+      (split_clocks(a, KC, smem, tiles, nsm) <= 1.02 * tile_clocks(a, BT, nsm) ||
+       (a.M + BT - 1) / BT > 65535)) {               // rows of plain_kernel's grid
     static std::atomic<uint64_t> granted{0};
     cudaError_t e = allow_smem(granted, plain_split_kernel<MW>, 232448);
     if (e != cudaSuccess) return cuda_fail(e, "plain kernel smem attribute");
     plain_split_kernel<MW><<<(unsigned)tiles, 32 * SWARPS, smem, s>>>(a, KC);
     return cuda_fail(cudaGetLastError(), "plain kernel launch");
   }
-  constexpr int BT = 16 * TH;
   dim3 grid((unsigned)((a.N + BT - 1) / BT), (unsigned)((a.M + BT - 1) / BT));
   plain_kernel<MW, TH><<<grid, 256, 0, s>>>(a);
   return cuda_fail(cudaGetLastError(), "plain kernel launch");
