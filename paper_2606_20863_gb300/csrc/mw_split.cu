@@ -531,7 +531,8 @@ bool exps_together(const SplitArgs &a, const SplitArgs &b, bool exponents_only) 
 }
 
 bool digits_together(const SplitArgs &a, const SplitArgs &b) {
-  return a.nmod == 0 && (a.R + b.R) * a.K <= kPairMaxEntries &&
+  // (the narrowest kernel for m = 16 takes 768 bits, also for a plan of fewer)
+  return a.nmod == 0 && a.m <= 8 && (a.R + b.R) * a.K <= kPairMaxEntries &&
          piece_bits(a.w, std::max(a.S, b.S)) <= kPairMaxBits;
 }
 

@@ -39,3 +39,14 @@ def test_wide_entries_that_fill_the_gpu(host, m, range_, n, ta, tb, two):
     p = host.plan(m, "ozaki", n, n, n, range_, range_)
     cuts = [l for l in host.launches(lambda: host.gemm(p, n, n, n, ta, tb)) if "pieces_" in l[0]]
     assert len(cuts) == 2 and (cuts[1][4] != 0) == two
+
+
+@pytest.mark.parametrize("m", [2, 4, 8, 16])
+@pytest.mark.parametrize("S", [1, 9, 20, 31, 32, 47])
+def test_plans_of_any_width(host, m, S):
+    # pieces a caller chose: m = 16 has no kernel for entries of up to 256 bits
+    p = host.plan(m, "ozaki", 16, 16, 16, 4, 4)
+    p.S_A, p.S_B, p.D = S, 1, S
+    for ta, tb in ((0, 0), (1, 0), (0, 1), (1, 1)):
+        cuts = [l for l in host.launches(lambda: host.gemm(p, 16, 16, 16, ta, tb)) if "pieces_" in l[0]]
+        assert len(cuts) == (1 if m < 16 and 8 * S + 3 <= 256 else 2)
