@@ -402,9 +402,10 @@ int launch_series_s(const DotArgs &a, cudaStream_t st) {
   // CTAs a series: all its rows, and with few series more, for the segments that are taken
   // by coefficients: two an SM while a series is short (40 octo-double series of 64
   // growing coefficients 185 -> 103 us), one an SM for longer ones, whose rows the exponent
-  // pass of idle CTAs would slow down (8 double-double series of 1,000: 46 -> 66 us)
+  // pass of idle CTAs would slow down (8 double-double series of 1,000: 46 -> 66 us);
+  // at most one a chunk's place (the kernel's `way` of a segment g starts at g + i0 / warps)
   const int ctas = (int)std::max<int64_t>((row_pairs + pairs - 1) / pairs,
-                                          std::min<int64_t>({a.K, (MW < 16 && a.K <= 256 ? 2 : 1) * nsm / a.count, 255}));
+                                          std::min<int64_t>({a.K + (a.K - 1) / (pairs * ks), (MW < 16 && a.K <= 256 ? 2 : 1) * nsm / a.count, 255}));
   const unsigned grid = (unsigned)std::min<int64_t>(a.count * ctas, 1 << 30);
   auto launch = [&](auto kernel, std::atomic<uint64_t> &granted) {
     cudaError_t e = allow_smem(granted, kernel, kSeriesSmem);
