@@ -387,16 +387,19 @@ int launch_series_s(const DotArgs &a, cudaStream_t st) {
   while (ks > 1 && smem_of(1, ks) > kSeriesSmem) ks /= 2;
   int pairs = std::min(row_pairs, kSeriesWarps / ks);
   while (pairs > 1 && smem_of(pairs, ks) > kSeriesSmem) --pairs;
-  // few rows for the SMs: coefficients one by one, for which warps count, not a row's share
-  if (a.count * row_pairs * 4 <= nsm)
-    for (int k = ks / 2; k >= 1; k /= 2) {
-      int p = std::min(row_pairs, kSeriesWarps / k);
-      while (p > 1 && smem_of(p, k) > kSeriesSmem) --p;
-      if (p * k > pairs * ks && smem_of(p, k) <= kSeriesSmem) {
-        ks = k;
-        pairs = p;
-      }
+  // few rows for the SMs: coefficients one by one, for which warps count, not a row's share;
+  // likewise where the sums of shared rows leave room for two or three warps only (8
+  // quad-double series of 2,000, growing: two warps 1,712 us, seven 474; from four warps
+  // on a row's share counts again, series of one magnitude 322 with four, 390 with eight)
+  const int least = a.count * row_pairs * 4 <= nsm ? pairs * ks + 1 : pairs * ks < 4 ? 4 : kSeriesWarps + 1;
+  for (int k = ks / 2; k >= 1; k /= 2) {
+    int p = std::min(row_pairs, kSeriesWarps / k);
+    while (p > 1 && smem_of(p, k) > kSeriesSmem) --p;
+    if (p * k >= least && p * k > pairs * ks && smem_of(p, k) <= kSeriesSmem) {
+      ks = k;
+      pairs = p;
     }
+  }
   const size_t smem = smem_of(pairs, ks);
   if (smem > kSeriesSmem) return fail(MW_EUNSUPPORTED, "series of %lld coefficients", (long long)a.K);
   // CTAs a series: all its rows, and with few series more, for the segments that are taken
@@ -429,12 +432,16 @@ int launch_series_m(int s_req, const DotArgs &a, cudaStream_t st) {
   }
 }
 
+// Digits in shared memory beside the columns of four warps.  With fewer a CTA, the only one
+// of its SM, is slower than the inner products where exponents grow (us, inner products /
+// one to three warps: 200 quad-double series of 2,100 33,230 / 74,390, 600 double-double
+// ones of 3,000 100,710 / 285,670, 76 octo-double ones of 1,150 9,310 / 12,020).
 template <int MW, int S>
 bool series_fits_m(int s_req, int64_t n) {
   if constexpr (S > DotS<MW>::hi) {
     return false;
   } else {
-    if (s_req == S) return n <= 4096 && series_smem<MW, S>(n, 1, 1) <= kSeriesSmem;
+    if (s_req == S) return n <= 4096 && series_smem<MW, S>(n, 4, 1) <= kSeriesSmem;
     return series_fits_m<MW, S + 1>(s_req, n);
   }
 }
