@@ -418,7 +418,7 @@ int mw_convolve_batched(const mw_plan *plan, int64_t count, int64_t n, const dou
   a.count = count; a.K = n; a.D = p.D; a.range_A = p.range_A; a.range_B = p.range_B;
   a.status = status_ptr();
   a.conv = 1;
-  if (series_fits(p.m, p.S_A, n)) return launch_series(p.m, p.S_A, a, (cudaStream_t)stream);
+  if (series_fits(p.m, p.S_A, count, n)) return launch_series(p.m, p.S_A, a, (cudaStream_t)stream);
   return launch_dot(p, a, (cudaStream_t)stream);
 }
 

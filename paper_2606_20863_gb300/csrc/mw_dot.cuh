@@ -35,9 +35,9 @@ template <> struct DotS<4> { static constexpr int lo = 8, hi = 12; };
 template <> struct DotS<8> { static constexpr int lo = 17, hi = 21; };
 template <> struct DotS<16> { static constexpr int lo = 35, hi = 36; };
 
-// Power series of n coefficients whose digits fit in shared memory (mw_series.cu);
-// false (nothing launched) when they do not: the inner-product kernel takes them.
-bool series_fits(int m, int S, int64_t n);
+// Whether mw_series.cu takes count power series of n coefficients: their digits fit in shared
+// memory and they are not so few that the inner-product kernel is the faster one.
+bool series_fits(int m, int S, int64_t count, int64_t n);
 int launch_series(int m, int S, const DotArgs &a, cudaStream_t st);
 
 namespace {

@@ -36,9 +36,10 @@
 //   dd 300 x 600      4,410 / 4,710 / 5,210 / 5,370      516 / 2,370 / 5,300 / 9,070   380 / 548 / 708 / 931
 //   od 40 x 64          179 / 183 / 189 / 193            39 / 199 / 398 / 585   25 / 48 / 76 / 103
 //   od 1 x 1,200        144 / 146 / 151 / 156            476 / 958 / 1,217 / 2,187   70 / 84 / 112 / 130
-//   od 1 x 128           21 / 21 / 23 / 23               31 / 150 / 325 / 562   17 / 19 / 21 / 25
-// (one to eight short double-double series growing by 45 binades in both operands stay
-// the exception: 12-19 us with one CTA a coefficient, 14-23 now).
+// So few coefficients that inner products fill the SMs once go there (one_wave).  Slower
+// than one CTA a coefficient were, growing by 45 binades in both operands, 12 octo-double
+// series of 24 (24.9 / 27.0; of one magnitude 22.8 / 14.3) and 4 double-double ones of 128
+// (18.7 / 20.9; 13.0 / 12.8).
 #include <cuda.h>
 
 #include <algorithm>
@@ -446,9 +447,23 @@ bool series_fits_m(int s_req, int64_t n) {
   }
 }
 
+// So few coefficients that a CTA each fills the SMs once: the inner products take the time
+// of one, the series kernel that of a chain of passes where exponents grow (us, inner
+// products / series kernel, series of one magnitude and growing by 45 binades: dd 1 x 200
+// 13.0 / 12.5 and 12.9 / 18.9, qd 1 x 128 12.7 / 12.5 and 13.6 / 18.8, 12 x 24 13.4 / 13.2
+// and 14.9 / 18.6, od 1 x 200 23.0 / 20.9 and 25.1 / 33.1; short octo-double series stay
+// with the series kernel, 1 x 64 18.7 / 14.2 and 20.7 / 20.8).
+bool one_wave(int m, int64_t count, int64_t n) {
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return m <= 4 ? count * n <= (m == 2 ? 3 : 2) * nsm : m == 8 && n > 64 && count * n <= 2 * nsm;
+}
+
 }  // namespace
 
-bool series_fits(int m, int S, int64_t n) {
+bool series_fits(int m, int S, int64_t count, int64_t n) {
+  if (one_wave(m, count, n)) return false;
   switch (m) {
     case 2: return series_fits_m<2, DotS<2>::lo>(S, n);
     case 4: return series_fits_m<4, DotS<4>::lo>(S, n);

@@ -1,6 +1,6 @@
-"""Which kernel multiplies power series, and with how many CTAs and warps: series
-whose digits leave room for the columns of fewer than four warps go to the inner-product
-kernel; growing exponents get
+"""Which kernel multiplies power series, and with how many CTAs and warps: so few
+coefficients that inner products fill the SMs once, and series whose digits leave room for
+the columns of fewer than four warps, go to the inner-product kernel; growing exponents get
 a CTA a coefficient without two of them sharing one.  The library's host code on a stand-in
 runtime of 152 SMs; no GPU."""
 import pytest
@@ -25,6 +25,10 @@ def launch(host, m, count, n, S):
 
 
 @pytest.mark.parametrize("m,count,n,S,kernel", [
+    (2, 1, 456, 7, "dot"), (2, 1, 457, 7, "series"), (2, 57, 8, 5, "dot"), (2, 58, 8, 5, "series"),
+    (4, 1, 304, 11, "dot"), (4, 1, 305, 11, "series"), (4, 12, 24, 10, "dot"), (4, 13, 24, 10, "series"),
+    (8, 1, 64, 20, "series"), (8, 1, 65, 20, "dot"), (8, 1, 304, 20, "dot"), (8, 1, 305, 20, "series"),
+    (8, 4, 64, 20, "series"), (16, 1, 64, 36, "series"), (16, 1, 200, 36, "series"),
     # digits beside four warps' columns, and beside three's
     (2, 600, 2944, 8, "series"), (2, 600, 3000, 8, "dot"), (4, 200, 2016, 12, "series"),
     (4, 200, 2050, 12, "dot"), (8, 76, 1120, 21, "series"), (8, 76, 1150, 21, "dot"),
