@@ -293,13 +293,13 @@ def timed(step, steps, flush, mw, dist, dev, phase=True):
 # is captured again.
 KERNEL_SOURCES = ("mw_ozaki.cu", "mw_tc.cuh", "mw_device.cuh", "mw_work.cuh")
 TRAFFIC = {
-    "qd1024": {"bytes": 394153216 + 85361664, "digest": "9ce880bc15265ecb"},
+    "qd1024": {"bytes": 393498112 + 85876992, "digest": "71d6980b23f5d6f6"},
     # 2,000 of the 20,000 products captured (the whole batch holds ~100 GB), x10
-    "od_batch": {"bytes": 10 * (2874157056 + 2759791616), "digest": "9ce880bc15265ecb"},
+    "od_batch": {"bytes": 10 * (2872154000 + 2760343000), "digest": "71d6980b23f5d6f6"},
     # residue form, captured at 2048^3 (quad double 64 moduli, double double 37) and
     # scaled by 4: residue planes in and residues out both grow with N^2
-    "qd4096_crt": {"bytes": 4 * (1073851648 + 508689920), "digest": "9ce880bc15265ecb"},
-    "dd4096_crt": {"bytes": 4 * (620855040 + 281017600), "digest": "9ce880bc15265ecb"},
+    "qd4096_crt": {"bytes": 4 * (1073901000 + 512438784), "digest": "71d6980b23f5d6f6"},
+    "dd4096_crt": {"bytes": 4 * (620879104 + 284281088), "digest": "71d6980b23f5d6f6"},
 }
 
 

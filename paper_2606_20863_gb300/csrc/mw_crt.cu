@@ -151,10 +151,12 @@ __device__ __forceinline__ bool in_range_bits(const uint32_t (&S)[NL], const uin
 // Kc = S + 1 rounded up to 16 (the K of the MMAs), whose constants are those of
 // column S-1.  The other columns q >= S multiply zero constants and may hold
 // anything finite.
-// Bound by the integer units (696 instructions a warp of entries before the last
-// trims, most of them selects, shifts and permutes; DRAM at half its rate), so the
-// words are placed by selects without branches, the sums reduced two moduli an
-// instruction (packed fp32), the range checked from the words' exponents, and only
+// Bound by the chain of a tile at three CTAs an SM (dependent integer instructions,
+// barriers around the shared tile, loads): 647 instructions a warp of entries, issue
+// slots 48 % busy, DRAM at 53 % (2048^2 quad doubles as stored, 146 us; stored K x N,
+// whose loads are 64 bytes of a row, 35 % and 39 %, 207 us).  So the words are placed by
+// selects without branches, the sums reduced two moduli an instruction (packed fp32), the
+// range checked from the words' exponents, and only
 // columns in use written and multiplied.  Both operands with their exponents, us,
 // before / now: 4096^2 quad doubles 1,658 / 1,320, double doubles 1,226 / 882.
 // Measured and left out: 64-byte rows of A for a fourth CTA an SM (1,465), residues
@@ -526,7 +528,8 @@ int launch_residues_nl(const SplitArgs &a, cudaStream_t s) {
 // them as they are.  One accumulator: a tile's product is issued when the previous
 // tile's sums have been read and runs while that tile is rounded; two buffers of
 // residues, the one just multiplied serving as the limb columns of the rounding
-// before its next load.  Bound by integer issue and latency: the kernel before this
+// before its next load.  Bound by the latency of a thread's chain of integer instructions
+// (issue slots 51 % busy, DRAM at 42 %): the kernel before this
 // (residues transposed through registers into a K-major A, two accumulators, X'
 // stored and read again for k) took 1,067 us for 4096^2 quad doubles, 781 us for
 // double doubles and 94 us for 777 x 1300 quad doubles; now 706, 527 and 72 us (with

@@ -19,7 +19,9 @@
 // S is a template parameter (digit positions known at compile time); the
 // planner picks the smallest instance that covers the error analysis.
 //
-// Bound by integer issue, the cut above all: 1,024 products of length 6,144, us,
+// Bound by the cut's integer instructions (ALU pipe 56 % busy at m = 2, where the exponent
+// pass before it waits for loads; 47 % at m = 8 with two CTAs an SM) and their latency:
+// 1,024 products of length 6,144, us,
 // before (64-bit limbs rounded up to pairs, range checked digit by digit, products
 // past the kept diagonals issued and masked) and now: m = 2 212 / 167, m = 4
 // 400 / 292, m = 8 603 / 500, m = 16 1,845 / 1,475 (L2 flushed).  128 threads a CTA:

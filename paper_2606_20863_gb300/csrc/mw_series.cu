@@ -27,7 +27,7 @@
 //
 // Bound by the 32 x 32 -> 64 bit multiply-adds (133 M warp instructions for 2,000
 // octo-double pairs of degree 127, about four cycles each and SM sub-partition:
-// 0.45 ms): those pairs take 0.62 ms, and took 17.25 ms with one CTA per coefficient
+// 0.45 ms, their pipe 77 % busy): those pairs take 0.62 ms, and took 17.25 ms with one CTA per coefficient
 // (which cuts i + 1 entries of both series again for each).  Exponents that grow along
 // the series cost more cuts.  us, entries growing by 0 / 20 / 45 binades in one operand /
 // 45 in both, with one CTA a coefficient, with rows alone, and now:
