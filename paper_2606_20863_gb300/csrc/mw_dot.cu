@@ -27,7 +27,8 @@
 // 400 / 292, m = 8 603 / 500, m = 16 1,845 / 1,475 (L2 flushed).  128 threads a CTA:
 // m = 2 195, m = 8 486; 5,000 products of length 500 148 -> 117, not taken.
 //
-// The same kernel multiplies truncated power series (mw_convolve_batched):
+// The same kernel multiplies the truncated power series that mw_series.cu does not take
+// (mw_convolve_batched, series_fits):
 // coefficient i of the product of series s, c_i = sum_{k<=i} a_k b_{i-k}, is the
 // inner product of a_0..a_i with b_i..b_0, so product u = (s, i) reads a forward
 // from a_0 and b backward from b_i, over i + 1 terms (Section 2's s_i are these
